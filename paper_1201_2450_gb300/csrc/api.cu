@@ -92,7 +92,7 @@ tnlm_status ensure_workspace(tnlm_geometry *g, bool need_tmp, long long n_scalar
 {
     ensure_coltab(g);
     const KGeom &kg = g->kg;
-    TNLM_TRY(dev_alloc(&g->d_r, (size_t)g->n_views_total * kg.npix));
+    TNLM_TRY(dev_alloc(&g->d_r, projection_floats(kg, g->n_views_total)));
     TNLM_TRY(dev_alloc(&g->d_g, (size_t)kg.np * kg.nvox));
     if (need_tmp) TNLM_TRY(dev_alloc(&g->d_tmp, (size_t)kg.np * kg.nvox));
     if (!g->d_part) {
@@ -1228,7 +1228,7 @@ tnlm_status tnlm_fdk(tnlm_geometry *geo, const float *proj, float *vol, void *st
     const KGeom &kg = geo->kg;
     if ((long long)kg.nz * kg.np > 65535) return arg_error("tnlm_fdk needs nz * n_phases <= 65535");
     if (kg.nu > 8192) return arg_error("tnlm_fdk needs nu <= 8192");
-    TNLM_TRY(dev_alloc(&geo->d_r, (size_t)geo->n_views_total * kg.npix));
+    TNLM_TRY(dev_alloc(&geo->d_r, projection_floats(kg, geo->n_views_total)));
     return launch_fdk(kg, geo->d_views, geo->d_view_off, geo->n_views_total, proj, geo->d_r, vol, as_stream(stream));
 }
 

@@ -28,8 +28,8 @@ struct KGeom {
     long long npix;          // nu*nv
     // launch shapes (defaults 4, 4, 8; chosen by tnlm_autotune)
     int fwd_by;              // projector shape: 2, 4, 8 (slab walker rows) or 102, 104, 108 (table walker)
-    int bp_by;               // band transpose block rows: 2 or 4
-    int bp_ch;               // band transpose z cells per thread: 4 or 8
+    int bp_by;               // band transpose: warps per block, 2 or 4
+    int bp_ch;               // band transpose z cells per thread: 4, or 8 (by size 8 or 16)
     // column tables of the table walker (owned by the geometry handle; null until built)
     const float2 *coltab;    // [views][coltab_kmax][nu]: (ray parameter leaving the xy cell, brick offset bits)
     int coltab_kmax;
@@ -93,7 +93,8 @@ tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_tot
 // vout = beta * vin + alpha * P^T proj.  scaled: proj already multiplied by
 // the ray length |source -> pixel| (the residual form written by mode 1).
 // pref_ws (nullable): prefix_floats() floats of workspace; when given and the
-// geometry allows it (bands_apply), the band/prefix-sum transpose runs.
+// geometry allows it (bands_apply), the band/prefix-sum transpose runs; a scaled proj then holds
+// projection_floats() floats (the residual workspace does).
 tnlm_status launch_backproject(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *proj,
                                const float *vin, float *vout, float alpha, float beta, bool scaled, float *pref_ws,
                                int n_views_total, cudaStream_t st);
@@ -107,6 +108,7 @@ tnlm_status launch_backproject(const KGeom &kg, const ViewGeom *views, const int
                                float *pref_ws, int n_views_total, cudaStream_t st);
 bool bands_apply(const KGeom &kg);
 size_t prefix_floats(const KGeom &kg, int n_views_total);
+size_t projection_floats(const KGeom &kg, int n_views_total);  // a projection set the scaled transpose may read
 
 tnlm_status launch_sweep(int nx, int ny, int nz, int np, const float *wsrc, const float *vals, const float *g,
                          float *out, int d, int M, float h, float mu, int clip, cudaStream_t st);

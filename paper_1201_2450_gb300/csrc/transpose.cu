@@ -14,7 +14,6 @@ namespace tnlm {
 namespace {
 
 constexpr int kBpBX = 32, kBpBY = 4, kBpCH = 8;  // exact transpose block: 32 x 4 columns, 8 voxels in z each
-// band transpose: 32 x BY columns (BY in {2, 4}), CH z cells per thread (CH in {4, 8})
 
 template <bool SCALED, class T>
 __global__ void __launch_bounds__(kBpBX *kBpBY)
@@ -191,39 +190,50 @@ __global__ void __launch_bounds__(256) k_colscan(KGeom G, const float *__restric
 }
 
 // Transpose for geometries where a ray's chord through one voxel column spans
-// at most two z cells.  For each view and pixel column iu, the rows of the
-// column chunk split into (i) band rows, whose chord crosses a z boundary
-// z_m: one exact crossing parameter splits the xy chord dg between cells m-1
-// and m; (ii) full rows between two bands, whose chord stays inside one cell:
-// they add r |D| dg each, summed by prefix sums (one prefix load per
-// boundary).  Equal to the per-cell exact tests of k_backproject up to
-// rounding.
+// at most two z cells.  For each view, pixel column iu and z boundary z_m, let
+//   B_m = sum over detector rows of r |D| (length of the row's chord below z_m);
+// cell m receives B_{m+1} - B_m.  The rows below L_m, the first row whose chord
+// may cross z_m, lie wholly below it, so B_m is the xy chord dg times one prefix
+// sum, plus the crossing rows' own shares: an exact clamp per row, 0 for a row
+// that turns out to lie above.  The boundary images at the near and far end of
+// the chord are less than one or two rows apart on most scanners (band_rows),
+// so the rows L_m (and L_m + 1) are the only candidates and a boundary needs no
+// loop and no test.
+// Equal to the per-cell exact tests of k_backproject up to rounding.
 //
+// A warp covers 8 x 4 voxel columns: whatever the view angle its lanes read
+// detector columns within ~12 voxels of each other (a row of 32 voxels spread
+// over 120 pixel columns when the rays run along y).  Rows are rounded up in
+// floating point (add a power of two with rounding up: the integer is in the
+// low mantissa bits) and addresses formed from those bits directly.
+constexpr int kBandWX = 8, kBandWY = 4;  // voxel columns of a warp
+constexpr float kRowMagic = 12582912.0f;                // 1.5 * 2^23: one unit per ulp
+constexpr long long kRowMagicBits = 0x4B400000LL;
+
 // One view of a thread's column chunk: every pixel column iu of the column's
 // footprint, each of its chord's cell boundaries in turn.
-template <int CH>
+// ROWS: candidate rows per boundary, 1 or 2, or 0 for any number (a loop).
+template <int CH, int ROWS>
 __device__ __forceinline__ void bands_view(const KGeom &G, const float4 *s_row, float c, float s, float xc, float yc,
-                                           int iz0, int nzc, float fvscale, float fvoff,
-                                           const float *__restrict__ pv, const float2 *__restrict__ ppv,
+                                           int iz0, const float *__restrict__ pv, const float2 *__restrict__ ppv,
                                            float (&acc)[CH])
 {
+    const float fvscale = G.inv_dv;
+    const float fvlo = G.vc - G.v_off * G.inv_dv - 1e-3f;  // row coordinate of v: v * fvscale + fvlo, less a margin
     const float a = xc * c + yc * s;   // view-frame coordinate toward the source
     const float b = -xc * s + yc * c;  // view-frame coordinate along u
-    const float ac = (G.sad - a) * G.inv_sdd;  // ray parameter at the column centre's depth
-    float umin = FLT_MAX, umax = -FLT_MAX;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float ex = (q & 1) ? G.hx : -G.hx, ey = (q & 2) ? G.hy : -G.hy;
-        const float ak = a + ex * c + ey * s;
-        const float bk = b - ex * s + ey * c;
-        const float uk = __fdividef(bk * G.sdd, G.sad - ak);  // footprint only (1e-3 px margin)
-        umin = fminf(umin, uk);
-        umax = fmaxf(umax, uk);
-    }
-    const float fu_lo = fmaxf((umin - G.u_off) * G.inv_du + G.uc - 1e-3f, -1.f);
-    const float fu_hi = fminf((umax - G.u_off) * G.inv_du + G.uc + 1e-3f, (float)G.nu);
-    const int iu_lo = max(0, (int)ceilf(fu_lo));
-    const int iu_hi = min(G.nu - 1, (int)floorf(fu_hi));
+    const float U = G.sad - a;
+    const float ac = U * G.inv_sdd;  // ray parameter at the column centre's depth
+    // u footprint: the column's half extent across the ray through its centre, at the nearest depth of its
+    // corners (a bound; pixel columns that miss the square drop out by their empty chord)
+    const float t = __fdividef(b, U);
+    const float ext = G.hx * fabsf(fmaf(t, c, -s)) + G.hy * fabsf(fmaf(t, s, c));
+    const float near = U - (G.hx * fabsf(c) + G.hy * fabsf(s));
+    const float fu = fmaf(t * G.sdd - G.u_off, G.inv_du, G.uc);
+    const float fw = __fdividef(ext * G.sdd, near) * G.inv_du + 2e-3f;
+    const int iu_lo = max(0, (int)ceilf(fmaxf(fu - fw, -1.f)));
+    const int iu_hi = min(G.nu - 1, (int)floorf(fminf(fu + fw, (float)G.nu)));
+    const int strideP = G.nu * (int)sizeof(float2), strideR = G.nu * (int)sizeof(float);
     for (int iu = iu_lo; iu <= iu_hi; ++iu) {
         const float u = ((float)iu - G.uc) * G.du + G.u_off;
         const float w = ac * u - b;
@@ -237,108 +247,110 @@ __device__ __forceinline__ void bands_view(const KGeom &G, const float4 *s_row, 
         if (!ok || !(glo < ghi)) continue;
         const float dg = ghi - glo;  // xy chord of this pixel column (ray-parameter units)
         const float sra = __fdividef(fvscale, ac + glo), srb = __fdividef(fvscale, ac + ghi);  // row maps (margin)
-        const float gmid = 0.5f * (glo + ghi);  // the chord's midpoint
-        const float *__restrict__ pc = pv + iu;
-        const float2 *__restrict__ pp = ppv + iu;
-        // first and last detector row of boundary zm's band (1e-3-row margins); the integer
-        // clamps where the rows are used keep every index inside the detector
-        auto band_rows = [&](float zm, int &lo_row, int &hi_row) {
-            const float pa = fmaf(zm, sra, fvoff), pb = fmaf(zm, srb, fvoff);
-            lo_row = __float2int_ru(fminf(pa, pb) - 1e-3f);
-            hi_row = __float2int_rd(fmaxf(pa, pb) + 1e-3f);
+        const float idg = __fdividef(1.f, dg);
+        const float cmid = 0.5f * (glo + ghi) * idg;  // the chord's midpoint in units of dg
+        const char *pr = reinterpret_cast<const char *>(pv + iu) - kRowMagicBits * strideR;
+        const char *pp = reinterpret_cast<const char *>(ppv + iu) - kRowMagicBits * strideP;
+        // share of row iv's chord below z = zm: the ray rises (v > 0) or falls (v < 0) through the crossing
+        // gs = (zm - ac v) / v, so the share is sat(sign(v) (gs - gmid) / dg + 1/2); a ray in the plane z = 0
+        // (v = 0, 1/|v| = inf) lies below every zm > 0 and above every zm <= 0 (half-open cells): +-inf, or NaN
+        // for zm = 0, saturate to 1 and 0; s_row[nv] and s_row[nv + 1] stand for no row: above every zm.  A row
+        // with no share adds nothing whatever its value (not read as 0 * inf; row nv is not a row of this view).
+        auto add_share = [&](float sum, int row, float zm, float r) {
+            const float4 rw = s_row[row];  // (v, 1/|v|, sign of v)
+            const float gs = fmaf(-ac, rw.x, zm) * rw.y;  // sign(v) gs
+            const float share = __saturatef(fmaf(gs, idg, fmaf(-rw.z, cmid, 0.5f)));
+            return share > 0.f ? fmaf(r, share, sum) : sum;
         };
-        // row images of boundary m at the near and far end of the xy chord; boundary m+1 is mapped
-        // one step ahead because the full rows of cell m end where its band begins.  The full rows
-        // of cell m and the band rows of boundary m together are the rows L_m .. L_{m+1} - 1,
-        // L_m = the first band row of boundary m clamped to [0, nv], so their sum is one prefix
-        // difference, from which the band rows' own values are taken off again.
-        float zm = fmaf((float)iz0, G.dz, G.b0z);
-        int blo_m, bhi_m;
-        band_rows(zm, blo_m, bhi_m);
-        float2 P_m = __ldg(pp + (long long)min(max(blo_m, 0), G.nv) * G.nu);
+        float hi_m = 0.f, lo_m = 0.f;  // B_m / dg as the prefix sum's high part and the rest
 #pragma unroll
         for (int m = 0; m <= CH; ++m) {
-            if (m > nzc) break;
-            const float zn = fmaf((float)(iz0 + m + 1), G.dz, G.b0z);
-            int blo_n, bhi_n;
-            band_rows(zn, blo_n, bhi_n);
-            // band rows of boundary m: split the chord at the crossing of z = zm.  A band is
-            // usually narrower than one detector row, so its first row is handled without a
-            // loop (predicated: the loads of all boundaries can be issued together) and any
-            // further rows by the loop after it.
-            const int r0 = max(0, blo_m), r1 = min(G.nv - 1, bhi_m);
-            float rband = 0.f;  // sum of the band rows' values
-            auto band_row = [&](int iv, bool on) {
-                const float4 rw = s_row[iv];  // (v, 1/|v|, sign of v)
-                float r = __ldg(pc + iv * G.nu);
-                r = on ? r : 0.f;  // a row outside the band adds nothing
-                rband += r;
-                // part of the chord below z = zm: the ray rises (v > 0) or falls (v < 0) through the
-                // crossing gs = (zm - ac v) / v, so below = clamp(sign(v) (gs - gmid) + dg / 2, 0, dg);
-                // a ray in the plane z = 0 (v = 0, 1/|v| = inf) lies below every zm > 0 and above
-                // every zm <= 0 (half-open cells): +-inf, or NaN for zm = 0, clamp to dg and 0
-                const float sgs = fmaf(-ac, rw.x, zm) * rw.y;  // sign(v) * gs
-                const float below = fminf(fmaxf(fmaf(0.5f, dg, fmaf(-rw.z, gmid, sgs)), 0.f), dg);
-                if (m > 0) acc[m - 1] = fmaf(r, below, acc[m - 1]);
-                if (m < nzc) acc[m] = fmaf(r, dg - below, acc[m]);
-            };
-            band_row(r0 <= r1 ? r0 : 0, r0 <= r1);
-            for (int iv = r0 + 1; iv <= r1; ++iv) band_row(iv, true);
-            // full rows of cell m: strictly between the bands of boundaries m and m+1
-            if (m < nzc) {
-                const float2 P_n = __ldg(pp + (long long)min(max(blo_n, 0), G.nv) * G.nu);
-                acc[m] = fmaf(((P_n.x - P_m.x) + (P_n.y - P_m.y)) - rband, dg, acc[m]);
-                P_m = P_n;
+            const float zm = fmaf((float)(iz0 + m), G.dz, G.b0z);
+            const float pa = fmaf(zm, sra, fvlo), pb = fmaf(zm, srb, fvlo);
+            const float lo = fmaxf(fminf(fminf(pa, pb), (float)G.nv), 0.f);
+            const int jb = __float_as_int(__fadd_ru(lo, kRowMagic));  // L_m, biased by kRowMagicBits
+            const float2 P = __ldg(reinterpret_cast<const float2 *>(pp + (long long)jb * strideP));
+            const float r = __ldg(reinterpret_cast<const float *>(pr + (long long)jb * strideR));
+            const int row = jb - (int)kRowMagicBits;
+            float rest = add_share(P.y, row, zm, r);
+            if (ROWS == 2) rest = add_share(rest, row + 1, zm, __ldg(reinterpret_cast<const float *>(pr + (long long)(jb + 1) * strideR)));
+            if (ROWS == 0) {  // further rows of a wider band
+                const int r1 = min(G.nv - 1, __float2int_rd(fmaxf(pa, pb) + 2e-3f));
+                for (int iv = row + 1; iv <= r1; ++iv) rest = add_share(rest, iv, zm, __ldg(pv + iu + (long long)iv * G.nu));
             }
-            zm = zn;
-            blo_m = blo_n;
-            bhi_m = bhi_n;
+            if (m > 0) acc[m - 1] = fmaf((P.x - hi_m) + (rest - lo_m), dg, acc[m - 1]);
+            hi_m = P.x;
+            lo_m = rest;
         }
     }
 }
 
-// Launch bounds: 36 warps per SM (9 blocks of 32 x 4 threads, 18 of 32 x 2), 56 registers per thread; at
-// 48 registers the band-row split spills.  The input is the ray-length-scaled residual (k_colscan writes a
-// scaled copy of an unscaled input).
-template <int CH, int BY, class T>
-__global__ void __launch_bounds__(kBpBX *BY, 36 / BY)
+// Resident warps per SM that the registers are budgeted for.  The 17 boundaries of 16 cells are one straight run
+// of independent gathers, and 128 registers let their loads be issued ahead: on the 10 x 256x256x64 workload 16
+// cells take 6.61 ms at 16 warps per SM, 7.5 at 20, 8.7 at 24; 8 cells 7.47 ms at 20 (7.8 at 16, 8.0 at 28).
+constexpr int bands_warps(int ch) { return ch == 16 ? 16 : 20; }
+
+// NW warps of 8 x 4 voxel columns, each thread CH z cells of one column.  SPLIT = 1: the warps lie side by side (two
+// along x) and each sums every view of the phase.  SPLIT = NW: the warps share one patch of columns, warp w takes the
+// views w, w + NW, ... and the partial sums are added in warp order: for volumes too small to fill the GPU otherwise.
+// The input is the ray-length-scaled residual (k_colscan writes a scaled copy of an unscaled input).  The chunk's
+// boundaries beyond the volume (ragged nz) are computed like the others and their cells not stored.
+// Bound by instruction issue (74 % of the slots, 22 instructions per boundary) with the L1's gathers behind it (67 %
+// of its wavefront rate); 2.7 times faster per boundary than row tests with min/max bounds on both ends of each band
+// and 32 x 1 column warps (k_backproject_bands at 10 x 256x256x64, 360 views x 512x384: 15.4 -> 6.5 ms).
+template <int CH, int NW, int SPLIT, int ROWS, class T>
+__global__ void __launch_bounds__(32 * NW, bands_warps(CH) / NW)
     k_backproject_bands(KGeom G, const ViewGeom *__restrict__ views, const int *__restrict__ view_off,
                         const float *__restrict__ proj, const float2 *__restrict__ pref, const T *vin,
                         T *vout, float alpha, float beta, int nchunks)
 {
-    constexpr int NT = kBpBX * BY;
+    static_assert(SPLIT == 1 || SPLIT == NW, "warps lie side by side or share one patch");
+    constexpr int NT = 32 * NW;
     extern __shared__ float4 sm4[];
-    float4 *s_row = sm4;  // per detector row: (v, 1/|v| or +inf, sign of v (+1 for v = 0), 0)
-    const int tid = threadIdx.y * kBpBX + threadIdx.x;
+    float4 *s_row = sm4;  // per detector row: (v, 1/|v| or +inf, sign of v (+1 for v = 0), 0); [nv], [nv + 1]: no row
+    const int tid = threadIdx.x;
     for (int t = tid; t < G.nv; t += NT) {
         const float v = ((float)t - G.vc) * G.dv + G.v_off;
         s_row[t] = make_float4(v, v != 0.f ? 1.0f / fabsf(v) : INFINITY, v < 0.f ? -1.f : 1.f, 0.f);
     }
+    if (tid < 2) s_row[G.nv + tid] = make_float4(1e30f, 1.f, 1.f, 0.f);
     __syncthreads();
-    const int ix = blockIdx.x * kBpBX + threadIdx.x;
-    const int iy = blockIdx.y * BY + threadIdx.y;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int px = SPLIT > 1 ? (int)blockIdx.x : (int)blockIdx.x * 2 + (warp & 1);
+    const int py = SPLIT > 1 ? (int)blockIdx.y : (int)blockIdx.y * (NW / 2) + (warp >> 1);
+    const int ix = px * kBandWX + (lane & (kBandWX - 1)), iy = py * kBandWY + lane / kBandWX;
     const int phase = blockIdx.z / nchunks;
     const int iz0 = (blockIdx.z % nchunks) * CH;
-    if (ix >= G.nx || iy >= G.ny) return;
-    const int nzc = min(CH, G.nz - iz0);
-    const float xc = G.b0x + ((float)ix + 0.5f) * G.dx;
-    const float yc = G.b0y + ((float)iy + 0.5f) * G.dy;
-    const float fvscale = G.inv_dv, fvoff = G.vc - G.v_off * G.inv_dv;  // row coordinate of v: v*fvscale + fvoff
+    bool inside = ix < G.nx && iy < G.ny;
+    if (SPLIT == 1 && !inside) return;
     float acc[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k) acc[k] = 0.f;
-
-    const int v_end = view_off[phase + 1];
-    for (int vg = view_off[phase]; vg < v_end; ++vg) {
-        const float c = views[vg].c, s = views[vg].s;
-        const float *__restrict__ pv = proj + (long long)vg * G.npix;
-        const float2 *__restrict__ ppv = pref + (long long)vg * (G.nv + 1) * G.nu;
-        bands_view<CH>(G, s_row, c, s, xc, yc, iz0, nzc, fvscale, fvoff, pv, ppv, acc);
+    if (inside) {
+        const float xc = G.b0x + ((float)ix + 0.5f) * G.dx;
+        const float yc = G.b0y + ((float)iy + 0.5f) * G.dy;
+        const int v_end = view_off[phase + 1];
+        for (int vg = view_off[phase] + (SPLIT > 1 ? warp : 0); vg < v_end; vg += SPLIT)
+            bands_view<CH, ROWS>(G, s_row, views[vg].c, views[vg].s, xc, yc, iz0, proj + (long long)vg * G.npix,
+                                  pref + (long long)vg * (G.nv + 1) * G.nu, acc);
+    }
+    if (SPLIT > 1) {
+        float *s_acc = reinterpret_cast<float *>(s_row + G.nv + 2);  // [NW - 1][CH][32]
+        if (warp > 0)
+#pragma unroll
+            for (int k = 0; k < CH; ++k) s_acc[((warp - 1) * CH + k) * 32 + lane] = acc[k];
+        __syncthreads();
+        inside = inside && warp == 0;
+        if (!inside) return;
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+            for (int w = 0; w < NW - 1; ++w) acc[k] += s_acc[(w * CH + k) * 32 + lane];
     }
     const long long base = (long long)phase * G.nvox + ((long long)iz0 * G.ny + iy) * G.nx + ix;
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
-        if (k < nzc) {
+        if (iz0 + k < G.nz) {
             const long long o = base + (long long)k * G.nx * G.ny;
             const float bp = alpha * acc[k];
             st_v(vout + o, beta != 0.f ? fmaf(beta, ld_v(vin + o), bp) : bp);
@@ -357,26 +369,94 @@ bool bands_apply(const KGeom &kg)
     return rise <= 0.9 * (double)kg.dz;
 }
 
+// The band transpose may read (and not use) the two rows after a view's last one, so a projection set it reads from is
+// allocated two rows longer.
+size_t projection_floats(const KGeom &kg, int n_views_total) { return (size_t)n_views_total * kg.npix + 2 * (size_t)kg.nu; }
+
 size_t prefix_floats(const KGeom &kg, int n_views_total)
 {
-    // (hi, lo) prefix sums plus a ray-length-scaled copy of an unscaled input
-    return (size_t)2 * n_views_total * (kg.nv + 1) * kg.nu + (size_t)n_views_total * kg.npix;
+    // (hi, lo) prefix sums plus a ray-length-scaled copy of an unscaled input (projection_floats)
+    return (size_t)2 * n_views_total * (kg.nv + 1) * kg.nu + projection_floats(kg, n_views_total);
 }
 
-template <int CH, int BY, class T>
+// Detector rows that a z boundary's images at the two ends of a chord through one voxel column may lie apart, as the
+// number of candidate rows (1, 2; 0: more), with the margins of bands_view: at depth U a chord of horizontal length
+// diag moves the image v of a boundary by at most |v| diag / U.  Images off the detector do not count (no rows there).
+static int band_rows(const KGeom &kg)
+{
+    const double x1 = fabs((double)kg.b0x), x2 = fabs((double)kg.b0x + (double)kg.nx * kg.dx);
+    const double y1 = fabs((double)kg.b0y), y2 = fabs((double)kg.b0y + (double)kg.ny * kg.dy);
+    const double z1 = fabs((double)kg.b0z), z2 = fabs((double)kg.b0z + (double)kg.nz * kg.dz);
+    const double near = (double)kg.sad - hypot(fmax(x1, x2), fmax(y1, y2));  // > 0: the volume lies inside the orbit
+    const double vmax = 0.5 * (kg.nv - 1) * (double)kg.dv + fabs((double)kg.v_off) + 2.0 * kg.dv;
+    const double v = fmin(fmax(z1, z2) * kg.sdd / near, vmax);
+    const double rows = v * hypot((double)kg.dx, (double)kg.dy) / (near * (double)kg.dv);
+    return rows <= 0.98 ? 1 : (rows <= 1.98 ? 2 : 0);
+}
+
+template <int CH, int NW, int SPLIT, int ROWS, class T>
+static tnlm_status launch_bands_m(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
+                                  const float2 *pref, const T *vin, T *vout, float alpha, float beta, cudaStream_t st)
+{
+    const int nchb = (kg.nz + CH - 1) / CH;
+    constexpr int TX = SPLIT > 1 ? kBandWX : 2 * kBandWX, TY = SPLIT > 1 ? kBandWY : (NW / 2) * kBandWY;
+    dim3 grid((kg.nx + TX - 1) / TX, (kg.ny + TY - 1) / TY, kg.np * nchb);
+    const size_t smem = sizeof(float4) * (kg.nv + 2) + (SPLIT > 1 ? sizeof(float) * (NW - 1) * CH * 32 : 0);
+    auto kern = k_backproject_bands<CH, NW, SPLIT, ROWS, T>;
+    if (smem > 48 * 1024)
+        TNLM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<grid, 32 * NW, smem, st>>>(kg, views, view_off, src, pref, vin, vout, alpha, beta, nchb);
+    TNLM_TRY_CUDA(cudaGetLastError());
+    return TNLM_OK;
+}
+
+// Wide bands run in one shape per form (the result does not depend on it): pixels that fine against the voxels are
+// rare, and the row loop, not the shape, sets their time.
+template <int CH, int NW, int SPLIT, class T>
 static tnlm_status launch_bands(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                 const float2 *pref, const T *vin, T *vout, float alpha, float beta, cudaStream_t st)
 {
-    const int nchb = (kg.nz + CH - 1) / CH;
-    dim3 grid((kg.nx + kBpBX - 1) / kBpBX, (kg.ny + BY - 1) / BY, kg.np * nchb);
-    const size_t smem = sizeof(float4) * kg.nv;
-    if (smem > 48 * 1024)
-        TNLM_TRY_CUDA(cudaFuncSetAttribute(k_backproject_bands<CH, BY, T>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_backproject_bands<CH, BY, T><<<grid, dim3(kBpBX, BY), smem, st>>>(kg, views, view_off, src, pref, vin, vout,
-                                                                               alpha, beta, nchb);
-    TNLM_TRY_CUDA(cudaGetLastError());
-    return TNLM_OK;
+    switch (band_rows(kg)) {
+    case 1: return launch_bands_m<CH, NW, SPLIT, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    case 2: return launch_bands_m<CH, NW, SPLIT, 2, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    default: return launch_bands_m<8, 4, SPLIT, 0, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    }
+}
+
+// Blocks of 16 x 8 voxel columns and ch cells
+static long long band_blocks(const KGeom &kg, int ch)
+{
+    return (long long)((kg.nx + 15) / 16) * ((kg.ny + 7) / 8) * kg.np * ((kg.nz + ch - 1) / ch);
+}
+
+// The form of the band transpose by size.  A launch fills the GPU from about one block per resident slot (152 SMs x 4
+// blocks).  Below that, with chunks of 8 cells, the four warps of a block split the views of one patch instead (4 x
+// 32^3, 20 views: stage 37 -> 25 us; 27 us in chunks of 4); the split depends on the geometry alone, so every launch
+// shape sums in the same order.  With bp_ch = 8 and bp_by = 4 (the defaults) the chunk is 16 cells where the volume has
+// them: a thread's chord set-up serves twice the cells (6.61 against 7.47 ms at 10 x 256x256x64), which padding an
+// odd number of 8-cell chunks must not eat up.
+constexpr long long kBandsFill = 152 * 4;
+
+template <class T>
+static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
+                                        const float2 *pref, const T *vin, T *vout, float alpha, float beta,
+                                        cudaStream_t st)
+{
+    if (band_blocks(kg, 8) < kBandsFill) {
+        if (kg.bp_ch == 8)
+            return launch_bands<8, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+        return launch_bands<4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    }
+    const int n8 = (kg.nz + 7) / 8;
+    if (kg.bp_ch == 8 && kg.bp_by == 4 && band_blocks(kg, 16) >= kBandsFill && (n8 % 2 == 0 || n8 > 8))
+        return launch_bands<16, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 8 && kg.bp_by == 4)
+        return launch_bands<8, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 8 && kg.bp_by == 2)
+        return launch_bands<8, 2, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 4 && kg.bp_by == 4)
+        return launch_bands<4, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    return launch_bands<4, 2, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
 }
 
 template <class T>
@@ -397,18 +477,11 @@ static tnlm_status launch_backproject_t(const KGeom &kg, const ViewGeom *views, 
             k_colscan<false><<<sg, 256, 0, st>>>(kg, proj, pref, rtil);
         TNLM_TRY_CUDA(cudaGetLastError());
         const float *src = scaled ? proj : rtil;
-        if (kg.bp_ch == 8 && kg.bp_by == 4)
-            TNLM_TRY((launch_bands<8, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st)));
-        else if (kg.bp_ch == 8 && kg.bp_by == 2)
-            TNLM_TRY((launch_bands<8, 2, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st)));
-        else if (kg.bp_ch == 4 && kg.bp_by == 4)
-            TNLM_TRY((launch_bands<4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st)));
-        else if (kg.bp_ch == 4 && kg.bp_by == 2)
-            TNLM_TRY((launch_bands<4, 2, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st)));
-        else {
+        if ((kg.bp_ch != 4 && kg.bp_ch != 8) || (kg.bp_by != 2 && kg.bp_by != 4)) {
             set_error("band transpose shape must be CH in {4, 8} and BY in {2, 4} (got %d, %d)", kg.bp_ch, kg.bp_by);
             return TNLM_ERR_ARG;
         }
+        TNLM_TRY(launch_bands_by_size<T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st));
         return TNLM_OK;
     }
     const size_t smem = sizeof(float4) * kg.nv + sizeof(float) * kBpCH * kBpBX * kBpBY;
