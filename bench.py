@@ -47,7 +47,7 @@ WORKLOAD = ("NCAT-shaped 4D TNLM-R FP32: 10 phases x 256x256x64 @ 2 mm, 36 views
 # measured on; a changed source invalidates the figure (reported as null).
 NCU_TRAFFIC = {
     # single-kernel captures on the 6-phase case of this workload, scaled by 10/6 to its 10 phases; the
-    # projector stage is the bricked copy plus the table walk, the transpose stage the column scan plus the bands
+    # projector stage is the z-fastest copy plus the table walk, the transpose stage the column scan plus the bands
     "k_forward": {"bytes_per_launch": int((100.727808e6 + 48.609024e6 + 606.395392e6 + 165.109504e6) * 10 / 6),
                   "source_sha": "4ee81dbf075d39bb"},
     "k_backproject": {"bytes_per_launch": int((169.919488e6 + 284.322560e6 + 556.931328e6 + 93.128448e6) * 10 / 6),
@@ -427,7 +427,7 @@ def run_ours(args, rank, world, local):
         "compute_peaks": cpk,
         "roofline": roofline,
         "clocks": clocks,
-        # per step: the projector stage (k_brick + k_forward_tab, or k_forward alone), the transpose stage
+        # per step: the projector stage (k_zfirst + k_forward_tab, or k_forward alone), the transpose stage
         # (k_colscan + k_backproject_bands on this workload), k_sweep_box
         "gpu_launches": int(stage_n[0] * (2 if k1_table else 1) + 2 * stage_n[1] + stage_n[2]),
         "e2e": {"value": round(e2e_value, 4), "unit": UNIT, "h2d_bytes_per_step": int(h2d),

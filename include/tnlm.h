@@ -114,7 +114,7 @@ tnlm_status tnlm_project(const tnlm_geometry *geom, const float *vol, float *pro
  * evaluated voxel-driven (each voxel gathers over the pixels whose rays cross
  * it), as used by the (P1) gradient of Eq. 5.  vol may hold garbage when
  * beta == 0.  Uses the handle's column prefix-sum workspace (cudaMalloc on
- * first use, 2 sum(n_views) (nv+1) nu + sum(n_views) nu nv floats; if that
+ * first use, 2 sum(n_views) (nv+1) nu + sum(n_views) nu nv + 2 nu floats; if that
  * allocation fails, or very thin slices make it inapplicable, the exact
  * per-cell form runs instead with the same results up to rounding), so calls
  * on one handle must not overlap on the GPU. */
@@ -392,14 +392,14 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
  * likewise), writing the chosen shape to *shape (nullable).
  * The projector shape is 2, 4 or 8 (the slab walker: blocks of 32 x that
  * many detector pixels, one ray per thread, each ray finding all its own
- * crossings) or 102, 104 or 108 (the table walker: blocks of 32 x 2, 4 or 8
- * pixels; the xy cells every detector column crosses are laid out once per
- * handle in device memory, views x (nx + ny + 2, rounded up to even) x nu
- * entries of 8 bytes, and each ray adds only its own z crossings, reading a
- * copy of the volume
- * that each projection first writes into the handle's workspace with its
- * z slices in 4 x 8 (x, y) bricks: N_p x nz x ceil(nx/4) x ceil(ny/8) x 32
- * voxels of 4 bytes, FP32 also for 16-bit storage).  A new handle starts at 104; its tables are built,
+ * crossings) or 102, 104 or 108 (the table walker: blocks of 4, 8 or 16
+ * detector columns x 64 rows; the xy cells every detector column crosses are
+ * laid out once per handle in device memory, views x nu x (nx + ny + 4,
+ * rounded up to even) entries of 8 bytes, and the rows of a column walk them
+ * together, adding their own z crossings, over a copy of the volume that
+ * each projection first writes into the handle's workspace z-fastest: N_p x
+ * ny x nx x nz voxels of 4 bytes, FP32 also for 16-bit storage; volumes of
+ * more than 2^20 slices run the slab walker).  A new handle starts at 104; its tables are built,
  * synchronising the device, by the first call that projects (or by
  * tnlm_set_launch_shapes), never during a stream capture; if the tables or
  * the copy cannot be allocated the slab walker with 4 rows runs.  The two

@@ -9,6 +9,8 @@
 // The ray parameter is measured in units of the source->pixel vector D
 // (chord = delta_parameter * |D|) and anchored at the isocentre plane so
 // that FP32 positions keep ~1e-5 voxel resolution.
+#include <type_traits>
+
 #include "ray_common.cuh"
 
 namespace tnlm {
@@ -166,32 +168,30 @@ __global__ void __launch_bounds__(kFwdBX *BY)
 // the detector row), so every row of the column crosses the same xy cells at
 // the same ray parameters.  k_coltab lays out that sequence once per
 // geometry handle -- entry k of (view, column): the ray parameter where the
-// ray leaves its k-th xy cell, and the cell's offset in a bricked z slice --
-// and k_forward_tab walks each row's ray through its column's entries,
-// adding only that row's z-plane crossings.  The walk has no branch on
-// in-plane crossings: the lanes of a warp are adjacent columns of one row,
-// each reading its own column's next entries (the tables interleave the
-// columns, so those reads are coalesced), and the z crossings, which depend
-// on the row alone, fall within an entry or two of each other across the
-// warp.  At one step the lanes' cells lie along a line across the rays, a
-// few cells long in x and y; in a slice stored x-fastest a warp's gather
-// then touches ~7 cache lines when the rays run along x, so the walker
-// reads a copy of the volume whose slices are stored in 4 x 8 (x, y) bricks
-// of 32 voxels, one 128-byte line each (~3 lines per gather, averaged over
-// view angles), which k_brick writes at the start of each projection.
+// ray leaves its k-th xy cell, and the offset of that cell's z run -- and
+// k_forward_tab walks the rows of a column through its entries together: a
+// warp is 32 adjacent rows of one column, so an entry is one value for the
+// whole warp and the rows' voxels are neighbours in z.  The walker reads a
+// copy of the volume stored z-fastest, which k_zfirst writes at the start of
+// each projection: 32 rows span a few voxels of one z run, one or two sectors
+// per gather where a row of 32 columns touched three cache lines.
 // ---------------------------------------------------------------------------
 
-constexpr int kColtabPad = 3;  // exit entry repeated after the last so reads ahead need no test
+constexpr int kColtabHead = 4;  // float2 before a column's entries: what the walk needs of the column, and its start
+constexpr int kColtabPad = 1;   // room after the last entry, so that entries can be read in pairs
+constexpr int kColtabAhead = 16;  // room after the last column: the walk reads up to two batches of entries ahead
 
-// Entries of one (view, column) are stored in pairs: pair j of column iu of view vg holds entries 2j, 2j+1 as
-// one float4 at float4 index (vg * kmax / 2 + j) * nu + iu (kmax even), so a warp's lanes read adjacent pairs.
-__host__ __device__ __forceinline__ long long coltab_slot(int vg, int e, int iu, int kmax, int nu)
+// Column iu of view vg: kmax consecutive float2 (kmax even: pairs are 16-byte aligned).  The head is
+//   [0] (ga, ha), [1] (gb, hb): planes of the two in-plane axes crossed before beta: floor(beta ga + ha), ...
+//   [2] (entries, as bits; their end), [3] (their start, unused)
+// and entry k stands at [kColtabHead + k].
+__host__ __device__ __forceinline__ long long coltab_base(int vg, int iu, int kmax, int nu)
 {
-    return (((long long)vg * (kmax >> 1) + (e >> 1)) * nu + iu) * 2 + (e & 1);
+    return ((long long)vg * nu + iu) * kmax;
 }
 
-// The in-plane part of the ray of detector column iu of view V, shared by
-// k_coltab and k_forward_tab (the same expressions as k_forward).
+// The in-plane part of the ray of detector column iu of view V (the same
+// expressions as k_forward).
 struct ColumnRay {
     float Dx, Dy, Ex, Ey, Gx, Gy, blo, bhi;
     bool ok;
@@ -246,11 +246,10 @@ struct ColumnRay {
     }
     __device__ __forceinline__ float beta_a(int m) const { return fmaf(fmaf((float)m, saf, fa0), iva, oa); }
     __device__ __forceinline__ float beta_b(int k) const { return fmaf(fmaf((float)k, sbf, fb0), ivb, ob); }
-    // offset of cell (a, b) in a bricked z slice (nxb = bricks along x)
-    __device__ __forceinline__ int cell(int ia, int ib, int nxb) const
+    // offset of cell (a, b)'s z run in a phase of the z-fastest volume
+    __device__ __forceinline__ int cell(const KGeom &G, int ia, int ib) const
     {
-        const int x = xa ? ia : ib, y = xa ? ib : ia;
-        return (((y >> 3) * nxb + (x >> 2)) << 5) + ((y & 7) << 2) + (x & 3);
+        return ((xa ? ib : ia) * G.nx + (xa ? ia : ib)) * G.nz;
     }
     // entries of the column: one per interior plane crossed, and the exit
     __device__ __forceinline__ int entries() const { return ok ? n_a + n_b + 1 : 0; }
@@ -259,10 +258,8 @@ struct ColumnRay {
 // Entries of every (view, column): thread t of (view vg, column iu) places the
 // t-th plane crossing (a-planes first, then b-planes) at its rank in the merged
 // order, found by binary search over the other axis (ties: the a-plane first);
-// the thread with t == n_a + n_b writes the exit, and repeats it in the next
-// kColtabPad slots so that the walk can read ahead without bounds tests.
-// Layout: pairs of entries interleaved by column (coltab_slot), kmax = nx + ny - 1 + kColtabPad rounded up to
-// an even count.
+// the thread with t == n_a + n_b writes the exit, thread 0 the head.
+// kmax = kColtabHead + nx + ny - 1 + kColtabPad rounded up to an even count.
 __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restrict__ views, float2 *__restrict__ tab,
                                                 int kmax)
 {
@@ -270,6 +267,13 @@ __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restr
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     ColumnRay R;
     R.init(G, views[vg], iu);
+    float2 *col = tab + coltab_base(vg, iu, kmax, G.nu);
+    if (t == 0) {
+        col[0] = make_float2(R.ok ? fabsf(R.Ga) : 0.f, R.ok ? (R.sa > 0 ? R.Ea - (float)R.ia0 : (float)(R.ia0 + 1) - R.Ea) : 0.f);
+        col[1] = make_float2(R.ok ? fabsf(R.Gb) : 0.f, R.ok ? (R.sb > 0 ? R.Eb - (float)R.ib0 : (float)(R.ib0 + 1) - R.Eb) : 0.f);
+        col[2] = make_float2(__int_as_float(R.entries()), R.bhi);
+        col[3] = make_float2(R.blo, 0.f);
+    }
     if (!R.ok || t > R.n_a + R.n_b) return;
     float beta;
     int e, ca, cb;
@@ -306,202 +310,299 @@ __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restr
         cb = R.ib0 + R.sb * k;
     }
     // the cell before this crossing; the crossing clamped to the column's extent
-    const float2 ent = make_float2(fminf(fmaxf(beta, R.blo), R.bhi), __int_as_float(R.cell(ca, cb, (G.nx + 3) >> 2)));
-    tab[coltab_slot(vg, e, iu, kmax, G.nu)] = ent;
-    if (t == R.n_a + R.n_b)
-        for (int q = 1; q <= kColtabPad; ++q) tab[coltab_slot(vg, e + q, iu, kmax, G.nu)] = ent;
+    col[kColtabHead + e] = make_float2(fminf(fmaxf(beta, R.blo), R.bhi), __int_as_float(R.cell(G, ca, cb)));
 }
 
+constexpr float kCellMagic = 12582912.0f;  // 1.5 * 2^23: one unit per ulp, so z + kCellMagic rounded down holds floor(z)
+constexpr int kCellMagicBits = 0x4B400000;
 
-// One ray per thread (block: 32 adjacent columns x BY rows of one view), walked
-// through its column's table two entries per step, the next two entries in
-// flight while the current pair is summed; a z crossing splits an entry's
-// segment (the loop takes any number of them, so no geometry condition
-// applies).
-// Launch bounds: 64 warps per SM (the walk is latency-bound on its voxel gathers, and full occupancy at 32
-// registers, with a few bytes spilled, beats 48 warps at 40 registers by 5 %).
-// vol: the bricked FP32 copy (widened from 16-bit storage by k_brick); y: the stored measurements.
-template <int MODE, int BY, class T>
-__global__ void __launch_bounds__(kFwdBX *BY, 64 / BY)
+// The entry of a column that holds beta, to rounding (h0: the first two of the column's head)
+__device__ __forceinline__ int entry_near(const float4 &h0, int K, float beta)
+{
+    const int na = __float_as_int(__fadd_rd(fmaf(beta, h0.x, h0.y), kCellMagic));
+    const int nb = __float_as_int(__fadd_rd(fmaf(beta, h0.z, h0.w), kCellMagic));
+    return min(max((na - kCellMagicBits) + (nb - kCellMagicBits), 0), K - 1);
+}
+
+// sum plus the parts that the walk of one row (z = ez + beta gz) took wrongly, one per z plane crossed between the
+// column's two ends; two planes at a time, so that their loads overlap.
+__device__ __forceinline__ float add_planes(const float4 *__restrict__ head, const float4 &h1,
+                                            const float *__restrict__ fp, int nz, float ez, float gz, float sum)
+{
+    const float2 *__restrict__ tc = reinterpret_cast<const float2 *>(head) + kColtabHead;
+    const int K = __float_as_int(h1.x);
+    const float blo = h1.z, bhi = h1.y, fnz = (float)nz;
+    const float za = fmaf(blo, gz, ez), zb = fmaf(bhi, gz, ez);
+    const int ia = (int)floorf(fminf(fmaxf(za, -1.f), fnz)), ib = (int)floorf(fminf(fmaxf(zb, -1.f), fnz));
+    const int n = abs(ib - ia);
+    if (n == 0) return sum;  // gz != 0 from here
+    const float4 h0 = __ldg(head);
+    const bool up = gz > 0.f;
+    const float iv = 1.0f / gz, ov = -ez * iv, stepf = up ? 1.f : -1.f;
+    const float p0 = (float)(up ? ia + 1 : ia);
+    for (int q = 0; q < n; q += 2) {
+        float pf[2], bp[2], e0[2];
+        float2 t[2];
+        int k[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            pf[i] = fmaf((float)(q + i), stepf, p0);
+            bp[i] = fminf(fmaxf(fmaf(pf[i], iv, ov), blo), bhi);
+            k[i] = entry_near(h0, K, bp[i]);
+            t[i] = __ldg(tc + k[i]);
+            e0[i] = __ldg(tc + k[i] - 1).x;
+        }
+        float diff[2];  // (voxel before plane p) - (voxel after)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            auto past = [&](float e) { return (fmaf(e, gz, ez) >= pf[i]) == up; };
+            while (k[i] > 0 && past(e0[i])) {
+                t[i] = __ldg(tc + --k[i]);
+                e0[i] = __ldg(tc + k[i] - 1).x;
+            }
+            while (k[i] < K - 1 && !past(t[i].x)) {
+                e0[i] = t[i].x;
+                t[i] = __ldg(tc + ++k[i]);
+            }
+            const int p = (int)pf[i];
+            const float *cp = fp + (__float_as_int(t[i].y) + p);  // the voxel above plane p
+            const float above = q + i < n && p < nz ? __ldg(cp) : 0.f, below = q + i < n && p > 0 ? __ldg(cp - 1) : 0.f;
+            diff[i] = up ? below - above : above - below;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            sum = q + i < n ? fmaf(diff[i], fminf(fmaxf(bp[i], e0[i]), t[i].x) - e0[i], sum) : sum;
+    }
+    return sum;
+}
+
+// A warp walks 32 R rows of one detector column (block: NC adjacent columns), R per lane, 32 apart.
+// Along an entry's segment e_{k-1} .. e_k a row stays in one voxel unless it crosses a z plane there, once in ~25
+// entries.  The walk takes every entry whole, with the voxel at its end:
+//   acc += (e_k - e_{k-1}) f(c_k, floor z(e_k)),   z(beta) = Ez + beta Gz, 0 outside the volume,
+// five operations per row and no test where all the warp's rows are inside, and add_planes then adds for every z
+// plane p of the row the part that this took wrongly:
+//   acc += (beta_p - e_{k-1}) (f(c_k, before p) - f(c_k, after p)),
+// k the first entry whose end lies past p, found from the planes crossed at beta_p (they number the entries) and
+// settled on the same z(e_k) that the walk used, so the two agree whatever the rounding.  The entry's voxels are
+// then split at beta_p exactly, any number of planes in one entry included, and a row that enters or leaves through
+// the top or bottom of the volume does so at plane 0 or nz.
+// vol: the z-fastest FP32 copy (widened from 16-bit storage by k_zfirst); y: the stored measurements.
+// Bound by the L1 (80 % of its data cycles: per entry one for each row's gather, and four for the 16 bytes of two
+// entries that every lane receives) with issue at 64 %: 17.1 G crossed voxels of 10 x 256x256x64, 360 views x
+// 512x384, in 8.3 ms, where a walk of 32 columns x 1 row that tested each entry for its plane took 10.8; 10 x 128^3,
+// 400 x 256x192 2.83 -> 1.47 ms.  Two rows per lane: each entry read serves both (1 row: 1.85 ms on the latter; 4
+// rows spill or leave too few warps).  32 warps per SM: the loads of two batches in flight want 64 registers (40
+// warps: 9.7 ms).
+template <int MODE, int NC, int R, class T>
+__global__ void __launch_bounds__(32 * NC, 32 / NC)
     k_forward_tab(KGeom G, const ViewGeom *__restrict__ views, const float *__restrict__ vol,
                   const T *__restrict__ y, float *__restrict__ out, double *__restrict__ partials)
 {
-    __shared__ double ws[BY];
-    const int iu = blockIdx.x * kFwdBX + threadIdx.x;
-    const int iv = blockIdx.y * BY + threadIdx.y;
-    const int vg = blockIdx.z;
-    double r2 = 0.0;
-    if (iu < G.nu && iv < G.nv) {
-        const ViewGeom V = views[vg];
-        ColumnRay R;
-        R.init(G, V, iu);
-        const float v = ((float)iv - G.vc) * G.dv + G.v_off;
-        const float Dz = v;
-        const float len = sqrtf(R.Dx * R.Dx + R.Dy * R.Dy + Dz * Dz);
-        const float Ez = (G.alpha0 * v - G.b0z) * G.inv_dz;
-        const float Gz = Dz * G.inv_dz;
-        float blo = R.blo, bhi = R.bhi;
-        bool ok = R.ok;
-        slab_grid(Ez, Gz, G.nz, blo, bhi, ok);
-        float acc = 0.f;
-        if (ok && blo < bhi) {
-            const int sc = Gz > 0.f ? 1 : -1;
-            const float ivc = Gz != 0.f ? 1.0f / Gz : 0.f, oc = -Ez * ivc, scf = (float)sc;
-            const int ic0 = clamp_floor(fmaf(blo, Gz, Ez), G.nz), ic1 = clamp_floor(fmaf(bhi, Gz, Ez), G.nz);
-            int nzc = Gz != 0.f ? abs(ic1 - ic0) : 0;  // z planes crossed inside the volume
-            float fc = (float)(ic0 + (Gz > 0.f));
-            float bc = nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
-            const long long zstep = sc * G.brick_slice;  // vol: the bricked copy
-            const float *__restrict__ fp = vol + ((long long)V.phase * G.nz + ic0) * G.brick_slice;
-            const long long st = G.nu;  // pair stride in the interleaved tables
-            const float2 *__restrict__ tc = G.coltab + coltab_slot(vg, 0, iu, G.coltab_kmax, G.nu);
-            auto entry_x = [&](int e) { return __ldg(tc + (long long)(e >> 1) * 2 * st + (e & 1)).x; };
-            const int K = R.entries();
-            // this row's entries: the first that ends after blo .. the first that ends at or after bhi
-            // (rows inside the volume's z range enter and leave through its sides: all entries)
-            int k0 = 0, k1 = K - 1;
-            if (blo > R.blo) {
-                int lo = 0, hi = K - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (entry_x(mid) > blo) hi = mid;
-                    else lo = mid + 1;
+    __shared__ float s_acc[32 * R][NC + 1];
+    __shared__ double ws[NC];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int row0 = blockIdx.y * 32 * R, vg = blockIdx.z;
+    const ViewGeom V = views[vg];
+    float acc[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[j] = 0.f;
+    const int iu_w = blockIdx.x * NC + w;
+    const float4 *__restrict__ head = reinterpret_cast<const float4 *>(
+        G.coltab + coltab_base(vg, iu_w < G.nu ? iu_w : 0, G.coltab_kmax, G.nu));
+    const float4 h0 = __ldg(head), h1 = __ldg(head + 1);
+    const int K = iu_w < G.nu ? __float_as_int(h1.x) : 0;
+    if (K > 0) {  // the same for the whole warp
+        const float2 *__restrict__ tc = reinterpret_cast<const float2 *>(head) + kColtabHead;  // tc[-1].x: the start
+        const float *__restrict__ fp = vol + (long long)V.phase * G.nvox;
+        const float fnz = (float)G.nz;
+        const float blo = h1.z, bhi = h1.y;
+        // where in beta any of the warp's rows is inside the volume (lo, hi), and where all are, by more than rounding
+        // could move a voxel (clo, chi)
+        float Ez[R], Gz[R];
+        float lo = FLT_MAX, hi = -FLT_MAX, clo = blo, chi = bhi;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const float v = ((float)min(row0 + 32 * j + lane, G.nv - 1) - G.vc) * G.dv + G.v_off;
+            Ez[j] = (G.alpha0 * v - G.b0z) * G.inv_dz;
+            Gz[j] = v * G.inv_dz;
+            const float za = fmaf(blo, Gz[j], Ez[j]), zb = fmaf(bhi, Gz[j], Ez[j]);
+            const float margin = fmaf(fabsf(Gz[j]), 1e-6f, 1e-3f);
+            if (fminf(za, zb) >= margin && fmaxf(za, zb) <= fnz - margin) {
+                lo = blo;
+                hi = bhi;
+            } else if (Gz[j] != 0.f) {
+                const float iv = 1.0f / Gz[j], m = margin * fabsf(iv);
+                const float t0 = -Ez[j] * iv, t1 = (fnz - Ez[j]) * iv;
+                const float jlo = fmaxf(blo, fminf(t0, t1)), jhi = fminf(bhi, fmaxf(t0, t1));
+                if (jlo < jhi) {
+                    lo = fminf(lo, jlo);
+                    hi = fmaxf(hi, jhi);
                 }
-                k0 = lo;
-            }
-            if (bhi < R.bhi) {
-                int lo = k0, hi = K - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (entry_x(mid) >= bhi) hi = mid;
-                    else lo = mid + 1;
-                }
-                k1 = lo;
-            }
-            float bcur = blo;
-            // one table entry (end e, cell offset c): its z crossings, then the rest of its segment
-            auto segment = [&](float e, float c) {
-                float f = ldg_v(fp + __float_as_int(c));
-                while (bc < e) {
-                    acc = fmaf(f, bc - bcur, acc);
-                    bcur = bc;
-                    fp += zstep;
-                    f = ldg_v(fp + __float_as_int(c));
-                    fc += scf;
-                    bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
-                }
-                acc = fmaf(f, e - bcur, acc);
-                bcur = e;
-            };
-            // entries before k1 end before bhi (the tables ascend), so only the last entry is clamped to
-            // the row's exit
-            const float4 *__restrict__ tp = reinterpret_cast<const float4 *>(tc) + (long long)(k0 >> 1) * st;
-            float4 t = __ldg(tp);
-            int k = k0;
-            if ((k & 1) && k < k1) {  // the first entry is the second of its pair
-                segment(t.z, t.w);
-                ++k;
-                tp += st;
-                t = __ldg(tp);
-            }
-            for (; k + 1 < k1; k += 2) {  // pairs of entries strictly before k1, the next pair in flight
-                tp += st;
-                const float4 n = __ldg(tp);
-                float f0 = ldg_v(fp + __float_as_int(t.y));
-                float f1 = ldg_v(fp + __float_as_int(t.w));
-                float e = t.x;
-                if (bc < e) {
-                    do {  // z crossings inside entry k's segment
-                        acc = fmaf(f0, bc - bcur, acc);
-                        bcur = bc;
-                        fp += zstep;
-                        f0 = ldg_v(fp + __float_as_int(t.y));
-                        fc += scf;
-                        bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
-                    } while (bc < e);
-                    f1 = ldg_v(fp + __float_as_int(t.w));
-                }
-                acc = fmaf(f0, e - bcur, acc);
-                bcur = e;
-                e = t.z;
-                while (bc < e) {  // z crossings inside entry k+1's segment
-                    acc = fmaf(f1, bc - bcur, acc);
-                    bcur = bc;
-                    fp += zstep;
-                    f1 = ldg_v(fp + __float_as_int(t.w));
-                    fc += scf;
-                    bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
-                }
-                acc = fmaf(f1, e - bcur, acc);
-                bcur = e;
-                t = n;
-            }
-            // the last one or two entries: k1 alone (k odd), or k (even) and then k1 if k < k1
-            if (k & 1) {
-                segment(fminf(t.z, bhi), t.w);
+                clo = fmaxf(clo, fminf(t0, t1) + m);
+                chi = fminf(chi, fmaxf(t0, t1) - m);
+            } else if (Ez[j] >= 0.f && Ez[j] < fnz) {  // in the plane of a face at most: tested voxel by voxel
+                lo = blo;
+                hi = bhi;
+                chi = -FLT_MAX;
             } else {
-                segment(fminf(t.x, bhi), t.y);
-                if (k < k1) segment(fminf(t.z, bhi), t.w);
+                chi = -FLT_MAX;
             }
         }
-        const float pf = acc * len;
+        int k0 = 0, k1 = K, c0 = 0, c1 = K;  // entries to walk, and of them those that need no test
+        if (!__all_sync(0xffffffffu, clo == blo && chi == bhi)) {
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                clo = fmaxf(clo, __shfl_xor_sync(0xffffffffu, clo, o));
+                chi = fminf(chi, __shfl_xor_sync(0xffffffffu, chi, o));
+            }
+            // two entries either side for the rounding of entry_near
+            k0 = lo < hi ? max(entry_near(h0, K, lo) - 2, 0) : 0;
+            k1 = lo < hi ? min(entry_near(h0, K, hi) + 3, K) : 0;
+            c0 = clo > blo ? max(entry_near(h0, K, clo) + 3, k0) : k0;
+            c1 = chi < bhi ? min(entry_near(h0, K, chi) - 2, k1) : k1;
+            if (!(clo < chi) || c0 >= c1) c0 = c1 = k1;
+        }
+        // entries k .. end - 1 of the rows; CHECKED: a voxel outside the volume counts 0
+        auto walk = [&](int k, int end, auto checked_tag) {
+            constexpr bool CHECKED = decltype(checked_tag)::value;
+            float prev = __ldg(tc + k - 1).x;
+            auto voxel = [&](float e, float c, int j) {
+                const int cell = __float_as_int(__fadd_rd(fmaf(e, Gz[j], Ez[j]), kCellMagic));
+                const float *q = fp + (unsigned)(__float_as_int(c) + cell - kCellMagicBits);
+                if (!CHECKED) return __ldg(q);
+                return (unsigned)(cell - kCellMagicBits) < (unsigned)G.nz ? __ldg(q) : 0.f;
+            };
+            auto single = [&](int k) {
+                const float2 t = __ldg(tc + k);
+#pragma unroll
+                for (int j = 0; j < R; ++j) acc[j] = fmaf(voxel(t.x, t.y, j), t.x - prev, acc[j]);
+                prev = t.x;
+            };
+            if ((k & 1) && k < end) single(k++);
+            int nb = (end - k) >> 2;  // batches of 4 entries
+            if (nb > 0) {
+                // the voxels of a batch are requested one batch, its table entries two batches ahead
+                const float4 *__restrict__ tp = reinterpret_cast<const float4 *>(tc + k);
+                k += 4 * nb;
+                float4 ta = __ldg(tp), tb = __ldg(tp + 1);
+                float f[4][R], seg[4];
+                auto request = [&] {
+                    const float e[4] = {ta.x, ta.z, tb.x, tb.z}, c[4] = {ta.y, ta.w, tb.y, tb.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < R; ++j) f[i][j] = voxel(e[i], c[i], j);
+                    seg[0] = e[0] - prev;
+                    seg[1] = e[1] - e[0];
+                    seg[2] = e[2] - e[1];
+                    seg[3] = e[3] - e[2];
+                    prev = e[3];
+                    tp += 2;
+                    ta = __ldg(tp);
+                    tb = __ldg(tp + 1);
+                };
+                request();
+#pragma unroll 2
+                for (; nb > 1; --nb) {
+                    float f0[4][R], seg0[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        seg0[i] = seg[i];
+#pragma unroll
+                        for (int j = 0; j < R; ++j) f0[i][j] = f[i][j];
+                    }
+                    request();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < R; ++j) acc[j] = fmaf(f0[i][j], seg0[i], acc[j]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < R; ++j) acc[j] = fmaf(f[i][j], seg[i], acc[j]);
+            }
+            for (; k < end; ++k) single(k);
+        };
+        if (k0 < c0) walk(k0, c0, std::true_type{});
+        if (c0 < c1) walk(c0, c1, std::false_type{});
+        if (c1 < k1) walk(c1, k1, std::true_type{});
+    }
+#pragma unroll
+    for (int j = 0; j < R; ++j) s_acc[32 * j + lane][w] = acc[j];
+    __syncthreads();
+    // Thread by (row, column) now, NC adjacent columns of a row together: the outputs are written so, and a plane is
+    // crossed by adjacent columns in neighbouring cells, by adjacent rows far apart (the gathers of the planes touch
+    // ~12 cache lines instead of 32).
+    double r2 = 0.0;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int t = threadIdx.x + 32 * NC * q;
+        const int iv = row0 + t / NC, iu = blockIdx.x * NC + t % NC;
+        if (iv >= G.nv || iu >= G.nu) continue;
+        const float u = ((float)iu - G.uc) * G.du + G.u_off;
+        const float v = ((float)iv - G.vc) * G.dv + G.v_off;
+        float sum = s_acc[t / NC][t % NC];
+        const float4 *__restrict__ head =
+            reinterpret_cast<const float4 *>(G.coltab + coltab_base(vg, iu, G.coltab_kmax, G.nu));
+        const float4 h1 = __ldg(head + 1);
+        if (__float_as_int(h1.x) > 0)
+            sum = add_planes(head, h1, vol + (long long)V.phase * G.nvox, G.nz, (G.alpha0 * v - G.b0z) * G.inv_dz,
+                             v * G.inv_dz, sum);
+        const float Dx = -G.sdd * V.c - u * V.s, Dy = -G.sdd * V.s + u * V.c;
+        const float len = sqrtf(Dx * Dx + Dy * Dy + v * v);
+        const float pf = sum * len;
         const long long o = ((long long)vg * G.nv + iv) * G.nu + iu;
         if (MODE == 0) {
             out[o] = pf;
         } else {
             const float r = pf - ldg_v(y + o);
             out[o] = r * len;  // scaled residual consumed by the transpose
-            r2 = (double)r * (double)r;
+            r2 += (double)r * (double)r;
         }
     }
     if (MODE == 1) {
-        const double s = block_sum_warps<BY>(r2, ws);
-        if (threadIdx.x == 0 && threadIdx.y == 0)
+        const double s = block_sum_warps<NC>(r2, ws);
+        if (threadIdx.x == 0)
             partials[((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
     }
 }
 
-// The bricked copy of the volume: thread t of z slice (phase, z) takes the
-// 4 x 2 voxels x = 4 bx .. 4 bx + 3, y = 2 py, 2 py + 1 and writes them as the
-// 8 consecutive elements they occupy in brick (bx, py / 4) (rows 2 py and
-// 2 py + 1 of a brick are adjacent), in FP32 whatever the stored type (16-bit
-// values are widened once here rather than at every gather of the walk).
-// Elements outside the volume are written as 0 and never read.
+// The z-fastest copy of the volume, [phase][y][x][z] in FP32 whatever the stored type (16-bit values are widened
+// once here rather than at every gather of the walk): tiles of 32 x by 32 z of one (phase, y) through shared memory.
 template <class T>
-__global__ void __launch_bounds__(256) k_brick(KGeom G, const T *__restrict__ vol, float *__restrict__ volb)
+__global__ void __launch_bounds__(256) k_zfirst(int nx, int ny, int nz, int ntx, int ntz, const T *__restrict__ vol,
+                                                float *__restrict__ volz)
 {
-    const int nxb = (G.nx + 3) >> 2, nyh = (G.ny + 1) >> 1;
-    const long long per_slice = (long long)nxb * nyh;
-    const long long n = per_slice * G.nz * G.np;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long sl = t / per_slice;  // phase * nz + z
-        const int r = (int)(t - sl * per_slice);
-        const int bx = r % nxb, py = r / nxb;
-        const T *src = vol + sl * G.nx * G.ny;
-        float v[8];
+    __shared__ float s[32][33];
+    long long b = blockIdx.x;
+    const int x0 = (int)(b % ntx) * 32;
+    b /= ntx;
+    const int z0 = (int)(b % ntz) * 32;
+    b /= ntz;
+    const int iy = (int)(b % ny);
+    const long long phase = b / ny, nvox = (long long)nx * ny * nz;
+    const int i = threadIdx.x & 31, r = threadIdx.x >> 5;
+    const T *src = vol + phase * nvox + (long long)iy * nx;
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+    for (int k = r; k < 32; k += 8)
+        if (x0 + i < nx && z0 + k < nz) s[k][i] = ld_v(src + (long long)(z0 + k) * ny * nx + x0 + i);
+    __syncthreads();
+    float *dst = volz + phase * nvox + (long long)iy * nx * nz;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int x = 4 * bx + i, y = 2 * py + j;
-                v[4 * j + i] = (x < G.nx && y < G.ny) ? ld_v(src + (long long)y * G.nx + x) : 0.f;
-            }
-        float *dst = volb + sl * G.brick_slice + ((((long long)(py >> 2) * nxb + bx) << 5) + ((py & 3) << 3));
-        reinterpret_cast<float4 *>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-        reinterpret_cast<float4 *>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
-    }
+    for (int k = r; k < 32; k += 8)
+        if (x0 + k < nx && z0 + i < nz) dst[(long long)(x0 + k) * nz + z0 + i] = s[i][k];
 }
 
 }  // namespace
 
-long long brick_slice(int nx, int ny) { return (long long)((nx + 3) / 4) * ((ny + 7) / 8) * 32; }
-
-size_t brick_bytes(const KGeom &kg) { return (size_t)kg.np * kg.nz * (size_t)kg.brick_slice * sizeof(float); }
+size_t volz_bytes(const KGeom &kg) { return (size_t)kg.np * kg.nvox * sizeof(float); }
 
 // Projector launch shape code: 2, 4 or 8 = the slab walker k_forward with blocks of 32 x that
-// many rows; 102, 104 or 108 = the table walker k_forward_tab with blocks of 32 x 2, 4 or 8 rows,
-// once the handle's column tables exist (else the slab walker with 4 rows).
+// many rows; 102, 104 or 108 = the table walker k_forward_tab with blocks of 4, 8 or 16 detector
+// columns, once the handle's column tables exist (else the slab walker with 4 rows).
 bool forward_shape_valid(int code)
 {
     return code == 2 || code == 4 || code == 8 || code == 102 || code == 104 || code == 108;
@@ -509,25 +610,37 @@ bool forward_shape_valid(int code)
 
 int forward_shape_in_use(const KGeom &kg)
 {
-    return (kg.fwd_by > 100 && !(kg.coltab && kg.volb)) ? 4 : kg.fwd_by;
+    return (kg.fwd_by > 100 && !(kg.coltab && kg.volz)) ? 4 : kg.fwd_by;
 }
+
+// Rows per lane of the table walker: two where the detector has them
+static int tab_rows(const KGeom &kg) { return kg.nv <= 32 ? 1 : 2; }
+
+static dim3 forward_grid(const KGeom &kg, int code, int n_views)
+{
+    if (code < 100) return dim3((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + code - 1) / code, n_views);
+    const int nc = 2 * (code - 100), rows = 32 * tab_rows(kg);
+    return dim3((kg.nu + nc - 1) / nc, (kg.nv + rows - 1) / rows, n_views);
+}
+
+static long long blocks_of(dim3 g) { return (long long)g.x * g.y * g.z; }
 
 long long forward_blocks(const KGeom &kg, int n_views_total)
 {
-    const int rows = forward_shape_in_use(kg) % 100;
-    return (long long)((kg.nu + kFwdBX - 1) / kFwdBX) * ((kg.nv + rows - 1) / rows) * n_views_total;
+    return blocks_of(forward_grid(kg, forward_shape_in_use(kg), n_views_total));
 }
 
 long long forward_blocks_max(const KGeom &kg, int n_views_total)
 {
-    return (long long)((kg.nu + kFwdBX - 1) / kFwdBX) * ((kg.nv + 1) / 2) * n_views_total;  // fewest rows: 2
+    const long long a = blocks_of(forward_grid(kg, 2, n_views_total)), b = blocks_of(forward_grid(kg, 102, n_views_total));
+    return a > b ? a : b;
 }
 
-int coltab_kmax(const KGeom &kg) { return (kg.nx + kg.ny - 1 + kColtabPad + 1) & ~1; }
+int coltab_kmax(const KGeom &kg) { return (kColtabHead + kg.nx + kg.ny - 1 + kColtabPad + 1) & ~1; }
 
 size_t coltab_entries(const KGeom &kg, int n_views_total)
 {
-    return (size_t)n_views_total * (size_t)coltab_kmax(kg) * (size_t)kg.nu;
+    return (size_t)n_views_total * (size_t)coltab_kmax(kg) * (size_t)kg.nu + kColtabAhead;
 }
 
 tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_total, float2 *tab, cudaStream_t st)
@@ -537,30 +650,45 @@ tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_tot
         set_error("column tables need nu <= 65535 (got %d)", kg.nu);
         return TNLM_ERR_ARG;
     }
-    dim3 grid((kmax + 127) / 128, kg.nu, n_views_total);
+    dim3 grid((kg.nx + kg.ny + 127) / 128, kg.nu, n_views_total);
     k_coltab<<<grid, 128, 0, st>>>(kg, views, tab, kmax);
     TNLM_TRY_CUDA(cudaGetLastError());
     return TNLM_OK;
 }
 
 template <int MODE, int BY, class T>
-static void launch_forward_by(const KGeom &kg, const ViewGeom *views, int n_views_total, const T *vol, const T *y,
+static void launch_forward_by(const KGeom &kg, const ViewGeom *views, int n_views, const T *vol, const T *y,
                               float *out, double *partials, cudaStream_t st)
 {
-    dim3 grid((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + BY - 1) / BY, n_views_total);
-    k_forward<MODE, BY, T><<<grid, dim3(kFwdBX, BY), 0, st>>>(kg, views, vol, y, out, partials);
+    k_forward<MODE, BY, T><<<forward_grid(kg, BY, n_views), dim3(kFwdBX, BY), 0, st>>>(kg, views, vol, y, out, partials);
 }
 
-template <int MODE, int BY, class T>
-static void launch_forward_tab(const KGeom &kg, const ViewGeom *views, int n_views_total, const T *vol, const T *y,
+// np phases of vol into the z-fastest copy
+template <class T>
+static void launch_zfirst(const KGeom &kg, int np, const T *vol, float *volz, cudaStream_t st)
+{
+    const int ntx = (kg.nx + 31) / 32, ntz = (kg.nz + 31) / 32;
+    k_zfirst<T><<<(unsigned)((long long)ntx * ntz * kg.ny * np), 256, 0, st>>>(kg.nx, kg.ny, kg.nz, ntx, ntz, vol, volz);
+}
+
+template <int MODE, int NC, class T>
+static void launch_walk(const KGeom &kg, const ViewGeom *views, int n_views, const float *volz, const T *y, float *out,
+                        double *partials, cudaStream_t st)
+{
+    const dim3 grid = forward_grid(kg, 100 + NC / 2, n_views);
+    if (tab_rows(kg) == 1)
+        k_forward_tab<MODE, NC, 1, T><<<grid, 32 * NC, 0, st>>>(kg, views, volz, y, out, partials);
+    else
+        k_forward_tab<MODE, NC, 2, T><<<grid, 32 * NC, 0, st>>>(kg, views, volz, y, out, partials);
+}
+
+template <int MODE, int NC, class T>
+static void launch_forward_tab(const KGeom &kg, const ViewGeom *views, int n_views, const T *vol, const T *y,
                                float *out, double *partials, cudaStream_t st)
 {
-    float *volb = static_cast<float *>(kg.volb);
-    const long long n = (long long)((kg.nx + 3) / 4) * ((kg.ny + 1) / 2) * kg.nz * kg.np;
-    const long long nb = (n + 255) / 256;
-    k_brick<T><<<(unsigned)(nb < 152 * 64 ? nb : 152 * 64), 256, 0, st>>>(kg, vol, volb);
-    dim3 grid((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + BY - 1) / BY, n_views_total);
-    k_forward_tab<MODE, BY, T><<<grid, dim3(kFwdBX, BY), 0, st>>>(kg, views, volb, y, out, partials);
+    float *volz = static_cast<float *>(kg.volz);
+    launch_zfirst<T>(kg, kg.np, vol, volz, st);
+    launch_walk<MODE, NC, T>(kg, views, n_views, volz, y, out, partials, st);
 }
 
 template <int MODE, class T>
@@ -570,9 +698,9 @@ static void launch_forward_mode(const KGeom &kg, const ViewGeom *views, int n_vi
     switch (forward_shape_in_use(kg)) {
     case 2: launch_forward_by<MODE, 2, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     case 8: launch_forward_by<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 102: launch_forward_tab<MODE, 2, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 104: launch_forward_tab<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 108: launch_forward_tab<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 102: launch_forward_tab<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 104: launch_forward_tab<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 108: launch_forward_tab<MODE, 16, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     default: launch_forward_by<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     }
 }
@@ -598,34 +726,9 @@ tnlm_status launch_forward(const KGeom &kg, const ViewGeom *views, int n_views_t
     return launch_forward_t<float>(kg, views, n_views_total, vol, y, out, partials, mode, st);
 }
 
-// One phase's share of a mode-1 projection: phase ph of vol is bricked (table walker) and views
+// One phase's share of a mode-1 projection: phase ph of vol is copied z-fastest (table walker) and views
 // [view_lo, view_hi) projected, writing the same rows of out and the same block partials as the
 // whole-volume launch does; the phases of a volume may so be projected as they arrive.
-template <int BY>
-static void launch_phase_by(const KGeom &kg, const ViewGeom *views, int ph, int view_lo, int view_hi, const float *vol,
-                            const float *y, float *out, double *partials, bool tab, cudaStream_t st)
-{
-    const int n = view_hi - view_lo;
-    const long long off = (long long)view_lo * kg.npix;
-    double *part = partials + (long long)view_lo * ((kg.nu + kFwdBX - 1) / kFwdBX) * ((kg.nv + BY - 1) / BY);
-    dim3 grid((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + BY - 1) / BY, n);
-    if (tab) {
-        float *volb = static_cast<float *>(kg.volb);
-        KGeom kb = kg;
-        kb.np = 1;
-        const long long nt = (long long)((kg.nx + 3) / 4) * ((kg.ny + 1) / 2) * kg.nz;
-        const long long nb = (nt + 255) / 256;
-        k_brick<float><<<(unsigned)(nb < 152 * 64 ? nb : 152 * 64), 256, 0, st>>>(
-            kb, vol + (long long)ph * kg.nvox, volb + (long long)ph * kg.nz * kg.brick_slice);
-        KGeom kt = kg;
-        kt.coltab = kg.coltab + (long long)view_lo * kg.coltab_kmax * kg.nu;
-        k_forward_tab<1, BY, float><<<grid, dim3(kFwdBX, BY), 0, st>>>(kt, views + view_lo, volb, y + off, out + off,
-                                                                         part);
-    } else {
-        k_forward<1, BY, float><<<grid, dim3(kFwdBX, BY), 0, st>>>(kg, views + view_lo, vol, y + off, out + off, part);
-    }
-}
-
 tnlm_status launch_forward_phase(const KGeom &kg, const ViewGeom *views, int ph, int view_lo, int view_hi,
                                  const float *vol, const float *y, float *out, double *partials, cudaStream_t st)
 {
@@ -635,12 +738,23 @@ tnlm_status launch_forward_phase(const KGeom &kg, const ViewGeom *views, int ph,
         return TNLM_ERR_ARG;
     }
     if (view_hi <= view_lo) return TNLM_OK;
-    const int code = forward_shape_in_use(kg);
-    const bool tab = code > 100;
-    switch (code % 100) {
-    case 2: launch_phase_by<2>(kg, views, ph, view_lo, view_hi, vol, y, out, partials, tab, st); break;
-    case 8: launch_phase_by<8>(kg, views, ph, view_lo, view_hi, vol, y, out, partials, tab, st); break;
-    default: launch_phase_by<4>(kg, views, ph, view_lo, view_hi, vol, y, out, partials, tab, st); break;
+    const int code = forward_shape_in_use(kg), n = view_hi - view_lo;
+    const long long off = (long long)view_lo * kg.npix;
+    const ViewGeom *vw = views + view_lo;
+    double *part = partials + blocks_of(forward_grid(kg, code, view_lo));
+    float *volz = static_cast<float *>(kg.volz);
+    KGeom kt = kg;
+    if (code > 100) {
+        launch_zfirst<float>(kg, 1, vol + (long long)ph * kg.nvox, volz + (long long)ph * kg.nvox, st);
+        kt.coltab = kg.coltab + (long long)view_lo * kg.coltab_kmax * kg.nu;
+    }
+    switch (code) {
+    case 2: launch_forward_by<1, 2, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
+    case 8: launch_forward_by<1, 8, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
+    case 102: launch_walk<1, 4, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
+    case 104: launch_walk<1, 8, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
+    case 108: launch_walk<1, 16, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
+    default: launch_forward_by<1, 4, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
     }
     TNLM_TRY_CUDA(cudaGetLastError());
     return TNLM_OK;

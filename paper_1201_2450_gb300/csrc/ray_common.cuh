@@ -77,6 +77,16 @@ __device__ __forceinline__ int clamp_floor(float x, int n)
     return (int)floorf(x);
 }
 
+// p + i size as one multiply-add.  Written out because the compiler otherwise gathers the terms of an address that
+// has several (the bias of an index held in a float's bits, and the row) into 64-bit sums and products of its own
+// (the band transpose at 10 x 256x256x64: 6.61 -> 6.39 ms).
+__device__ __forceinline__ const char *at(const char *p, int i, int size)
+{
+    const char *q;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(q) : "r"(i), "r"(size), "l"(p));
+    return q;
+}
+
 // sum over a block of NW warps (fixed order)
 template <int NW>
 __device__ __forceinline__ double block_sum_warps(double v, double *ws)

@@ -31,13 +31,11 @@ struct KGeom {
     int bp_by;               // band transpose: warps per block, 2 or 4
     int bp_ch;               // band transpose z cells per thread: 4, or 8 (by size 8 or 16)
     // column tables of the table walker (owned by the geometry handle; null until built)
-    const float2 *coltab;    // [views][coltab_kmax][nu]: (ray parameter leaving the xy cell, brick offset bits)
+    const float2 *coltab;    // [views][nu][coltab_kmax]: (ray parameter leaving the xy cell, z run offset bits)
     int coltab_kmax;
-    // the table walker's copy of the volume, each z slice laid out in 4 x 8 (x, y) bricks of 32
-    // voxels (x fastest inside a brick, bricks x-major): [N_p][nz][brick_slice] elements of the
-    // projected volume's type, written by the projector launch itself (null until built)
-    void *volb;
-    long long brick_slice;   // ceil(nx / 4) * ceil(ny / 8) * 32
+    // the table walker's FP32 copy of the volume, z fastest: [N_p][ny][nx][nz], written by the
+    // projector launch itself (null until built)
+    void *volz;
 };
 
 // One projection view: rotation and owning phase.
@@ -86,8 +84,7 @@ int forward_shape_in_use(const KGeom &kg);  // the code that runs: the slab walk
 // column tables of the table walker: entries per view and column (nx + ny - 1 + padding), total, build
 int coltab_kmax(const KGeom &kg);
 size_t coltab_entries(const KGeom &kg, int n_views_total);
-long long brick_slice(int nx, int ny);  // elements of one bricked z slice
-size_t brick_bytes(const KGeom &kg);    // the bricked copy of the N_p phases at 4 bytes per voxel
+size_t volz_bytes(const KGeom &kg);     // the z-fastest copy of the N_p phases at 4 bytes per voxel
 tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_total, float2 *tab, cudaStream_t st);
 
 // vout = beta * vin + alpha * P^T proj.  scaled: proj already multiplied by
@@ -272,7 +269,7 @@ struct tnlm_geometry {
     double *d_scalars = nullptr;      // reduction results
     float *d_pref = nullptr;          // column prefix sums for the transpose (prefix_floats)
     float2 *d_coltab = nullptr;       // column tables of the table projector (coltab_entries)
-    void *d_volb = nullptr;           // its bricked volume copy (brick_bytes)
+    void *d_volz = nullptr;           // its z-fastest volume copy (volz_bytes)
     // host-buffer entry point: a copy stream and one event per phase (created on first use)
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t copy_start = nullptr;
@@ -299,7 +296,7 @@ namespace tnlm {
 // the band-transpose prefix array (nullptr when the geometry does not admit
 // that transpose or the allocation failed).
 tnlm_status ensure_workspace(tnlm_geometry *g, bool need_tmp, long long n_scalars);
-// Column tables of the table projector and its bricked volume copy: built and
+// Column tables of the table projector and its z-fastest volume copy: built and
 // allocated on first use (synchronising the device, so never during stream
 // capture); on allocation failure the slab walker runs instead (the same
 // model, FP32 rounding of its own).

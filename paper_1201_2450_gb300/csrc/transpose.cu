@@ -269,11 +269,11 @@ __device__ __forceinline__ void bands_view(const KGeom &G, const float4 *s_row, 
             const float pa = fmaf(zm, sra, fvlo), pb = fmaf(zm, srb, fvlo);
             const float lo = fmaxf(fminf(fminf(pa, pb), (float)G.nv), 0.f);
             const int jb = __float_as_int(__fadd_ru(lo, kRowMagic));  // L_m, biased by kRowMagicBits
-            const float2 P = __ldg(reinterpret_cast<const float2 *>(pp + (long long)jb * strideP));
-            const float r = __ldg(reinterpret_cast<const float *>(pr + (long long)jb * strideR));
+            const float2 P = __ldg(reinterpret_cast<const float2 *>(at(pp, jb, strideP)));
+            const float r = __ldg(reinterpret_cast<const float *>(at(pr, jb, strideR)));
             const int row = jb - (int)kRowMagicBits;
             float rest = add_share(P.y, row, zm, r);
-            if (ROWS == 2) rest = add_share(rest, row + 1, zm, __ldg(reinterpret_cast<const float *>(pr + (long long)(jb + 1) * strideR)));
+            if (ROWS == 2) rest = add_share(rest, row + 1, zm, __ldg(reinterpret_cast<const float *>(at(pr, jb + 1, strideR))));
             if (ROWS == 0) {  // further rows of a wider band
                 const int r1 = min(G.nv - 1, __float2int_rd(fmaxf(pa, pb) + 2e-3f));
                 for (int iv = row + 1; iv <= r1; ++iv) rest = add_share(rest, iv, zm, __ldg(pv + iu + (long long)iv * G.nu));
