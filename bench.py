@@ -61,7 +61,7 @@ def _src_sha(fname: str) -> str:
     return hashlib.sha256(open(p, "rb").read()).hexdigest()[:16]
 
 
-KERNEL_SRC = {"k_forward": "projector.cu", "k_backproject": "transpose.cu", "k_sweep": "sweep_box.cuh"}
+KERNEL_SRC = {"k_forward": "projector.cu", "k_backproject": "transpose.cu", "k_sweep": "sweep_tile.cuh"}
 
 
 def measured_peaks() -> dict:

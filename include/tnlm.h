@@ -375,9 +375,10 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
 
 /* Launch-shape autotuning (no counterpart in the paper; it serves speed
  * only).  Several launch shapes of the hot kernels are compiled: projector
- * blocks of 32 x {2,4,8} pixels, band-transpose blocks of 32 x {2,4} voxel
- * columns with {4,8} z cells per thread, and 4 warp layouts of the box-sum
- * sweep.  Every shape computes each output with the same operations in the
+ * blocks of {4,8,16} detector columns (the slab walker: 32 x {2,4,8} pixels),
+ * band-transpose blocks of 8 x {8,16} voxel columns with 4, or 8 or 16, z
+ * cells per thread, and the warp layouts of the box-sum sweep (codes 0 and 2
+ * are one, 1 and 3 the other).  Every shape computes each output with the same operations in the
  * same order, so results do not depend on the choice.
  * tnlm_autotune times each shape on the handle's problem size (synthetic
  * inputs in stream-ordered scratch, one warm-up and the best of two timed

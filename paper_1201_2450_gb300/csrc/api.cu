@@ -696,14 +696,14 @@ static bool grouped_applies(int n, const tnlm_params *params)
 static tnlm_status prepare_grouped(int n, tnlm_geometry *const *geoms, float *const *f, const tnlm_params *params,
                                    void **mem, long long *total)
 {
-    const int d = params[0].d, M = params[0].M, v = box_shape(d, M, 0);
+    const int d = params[0].d, M = params[0].M;
     std::vector<GroupSweep> h((size_t)n);
     long long first = 0;
     for (int b = 0; b < n; ++b) {
         const KGeom &kg = geoms[b]->kg;
         GroupSweep &q = h[(size_t)b];
         long long items = 0;
-        box_grouped_tiles(v, d, M, kg.nx, kg.ny, kg.nz, kg.np, &q.ntx, &q.nty, &q.ntz, &items);
+        box_grouped_tiles(d, M, kg.nx, kg.ny, kg.nz, kg.np, &q.ntx, &q.nty, &q.ntz, &items);
         q.wsrc = q.vals = q.g = geoms[b]->d_g;
         q.out = f[b];
         q.nx = kg.nx;
@@ -785,8 +785,7 @@ static tnlm_status capture_batch(int n, tnlm_geometry *const *geoms, const T *co
             auto *counter = reinterpret_cast<unsigned long long *>(static_cast<GroupSweep *>(*group_mem) + n);
             cuda_ok(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), cs), "cudaMemsetAsync");
             cudaError_t err = cudaSuccess;
-            launch_box_grouped(box_shape(params[0].d, params[0].M, 0), params[0].d, params[0].M, probs, n, total,
-                               counter, sms, cs, &err);
+            launch_box_grouped(params[0].d, params[0].M, probs, n, total, counter, sms, cs, &err);
             cuda_ok(err, "grouped sweep launch");
         }
         cudaGraph_t gr = nullptr;

@@ -14,7 +14,7 @@
 // near a fixed point of Eq. 8 (f close to its weighted means) the gradient is
 // small against f and a form such as f (1 + sum w) - sum w f_j would lose the
 // digits that matter.
-#include "sweep_box.cuh"
+#include "box_block.cuh"
 
 namespace tnlm {
 namespace box {

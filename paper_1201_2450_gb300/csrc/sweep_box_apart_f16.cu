@@ -1,0 +1,5 @@
+// The box-sum sweep on FP16 images with values apart from the weights' sources.
+#include "sweep_box.cuh"
+
+TNLM_BOX_ENTRY(launch_box_apart_big, kBig, false, __half)
+TNLM_BOX_ENTRY(launch_box_apart_small, kSmall, false, __half)

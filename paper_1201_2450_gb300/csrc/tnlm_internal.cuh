@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libtnlm.so.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -207,14 +208,17 @@ struct GroupSweep {
     float c2, mu;
     int clip;
 };
-bool launch_box_grouped(int v, int d, int M, const GroupSweep *probs, int nprob, long long total,
-                        unsigned long long *counter, int sms, cudaStream_t st, cudaError_t *err);
-bool box_grouped_tiles(int v, int d, int M, int nx, int ny, int nz, int np, int *ntx, int *nty, int *ntz,
-                       long long *items);
+bool launch_box_grouped(int d, int M, const GroupSweep *probs, int nprob, long long total, unsigned long long *counter,
+                        int sms, cudaStream_t st, cudaError_t *err);
+bool box_grouped_tiles(int d, int M, int nx, int ny, int nz, int np, int *ntx, int *nty, int *ntz, long long *items);
 
-// Box-sum sweep launch shapes (sweep_box.cuh); each returns false when (d, M)
-// has no box kernel.  box_shape / set_box_shape hold the process-wide choice
-// per (d, M, storage) that tnlm_autotune makes.
+// Volumes that sweep with the smaller block (sweep_box.cuh has both sides' times).  By the volume alone, so that the
+// phases of a sharded or grouped call and every launch shape sum alike.
+__host__ __device__ inline bool sweep_small(int nx, int ny, int nz) { return (long long)nx * ny * nz <= 600000; }
+
+// Box-sum sweep launch shapes: 0 and 2 are one, 1 and 3 the other of two (big volumes, FP32 images; the others have
+// one).  launch_box_shape returns false when (d, M) has no box kernel.  box_shape / set_box_shape hold the
+// process-wide choice per (d, M, storage) that tnlm_autotune makes.
 constexpr int kBoxShapes = 4;
 // storage: 0 FP32, 1 BF16, 2 FP16 (a nonzero value other than 2 reads as BF16)
 int box_shape(int d, int M, int storage);
@@ -228,24 +232,19 @@ bool launch_box_shape_bf16(int v, int d, int M, int nx, int ny, int nz, int np, 
 bool launch_box_shape_f16(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const __half *wsrc,
                           const __half *vals, const __half *g, __half *out, float c2, float mu, int clip,
                           cudaStream_t st, cudaError_t *err);
-#define TNLM_BOX_DECL(V)                                                                                          \
-    bool launch_box_var##V(int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const float *wsrc,     \
-                           const float *vals, const float *g, float *out, float c2, float mu, int clip,          \
-                           cudaStream_t st, cudaError_t *err);                                                    \
-    bool launch_box_var##V##_bf16(int d, int M, int nx, int ny, int nz, int np, int p0, int nout,                \
-                                  const uint16_t *wsrc, const uint16_t *vals, const uint16_t *g, uint16_t *out,   \
-                                  float c2, float mu, int clip, cudaStream_t st, cudaError_t *err);              \
-    bool launch_box_var##V##_f16(int d, int M, int nx, int ny, int nz, int np, int p0, int nout,                 \
-                                 const __half *wsrc, const __half *vals, const __half *g, __half *out, float c2,  \
-                                 float mu, int clip, cudaStream_t st, cudaError_t *err);                          \
-    bool launch_box_grouped_var##V(int d, int M, const GroupSweep *probs, int nprob, long long total,            \
-                                   unsigned long long *counter, int sms, cudaStream_t st, cudaError_t *err);      \
-    bool box_grouped_tiles_var##V(int d, int M, int nx, int ny, int nz, int np, int *ntx, int *nty, int *ntz,     \
-                                  long long *items);
-TNLM_BOX_DECL(0)
-TNLM_BOX_DECL(1)
-TNLM_BOX_DECL(2)
-TNLM_BOX_DECL(3)
+#define TNLM_BOX_DECL(NAME, T)                                                                                       \
+    bool NAME(int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const T *wsrc, const T *vals, const T *g, \
+              T *out, float c2, float mu, int clip, cudaStream_t st, cudaError_t *err);
+#define TNLM_BOX_DECLS(T)                  \
+    TNLM_BOX_DECL(launch_box_big, T)       \
+    TNLM_BOX_DECL(launch_box_small, T)     \
+    TNLM_BOX_DECL(launch_box_apart_big, T) \
+    TNLM_BOX_DECL(launch_box_apart_small, T)
+TNLM_BOX_DECLS(float)
+TNLM_BOX_DECLS(__nv_bfloat16)
+TNLM_BOX_DECLS(__half)
+TNLM_BOX_DECL(launch_box_big2, float)
+#undef TNLM_BOX_DECLS
 #undef TNLM_BOX_DECL
 
 }  // namespace tnlm

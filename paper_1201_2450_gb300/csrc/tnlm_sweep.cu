@@ -1,6 +1,6 @@
 // TNLM step of the method: the patch-similarity weights of Eq. 9 fused into
-// one Gauss-Jacobi sweep of Eq. 8.  The box-sum kernels (sweep_box.cuh, one
-// translation unit per launch shape) cover d in {1,2}, M in {1,2,3}; this
+// one Gauss-Jacobi sweep of Eq. 8.  The box-sum kernels (sweep_box.cuh, the
+// sweep_box_*.cu units) cover d in {1,2}, M in {1,2,3}; this
 // file holds the direct tiled form for the other (d, M) (k_sweep), the
 // explicit export of the normalised weights (k_weights), the launch-shape
 // table and the sweep launchers.
@@ -16,6 +16,7 @@
 // kRescale, so no weight overflows and the largest weight is >= 1.
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "tnlm_internal.cuh"
 
@@ -196,28 +197,45 @@ void set_box_shape(int d, int M, int storage, int v)
     g_box_shape[d][M][storage_index(storage)] = v;
 }
 
+template <class T>
+static bool launch_box_t(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const T *wsrc,
+                         const T *vals, const T *g, T *out, float c2, float mu, int clip, cudaStream_t st,
+                         cudaError_t *err)
+{
+    const bool small = sweep_small(nx, ny, nz);
+    if (vals != wsrc && small)
+        return launch_box_apart_small(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
+    if (vals != wsrc)
+        return launch_box_apart_big(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
+    if (small) return launch_box_small(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
+    if constexpr (std::is_same<T, float>::value) {
+        if (v & 1) return launch_box_big2(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
+    }
+    return launch_box_big(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
+}
+
 bool launch_box_shape(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const float *wsrc,
                       const float *vals, const float *g, float *out, float c2, float mu, int clip, cudaStream_t st,
                       cudaError_t *err)
 {
-    switch (v) {
-    case 1: return launch_box_var1(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 2: return launch_box_var2(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 3: return launch_box_var3(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    default: return launch_box_var0(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    }
+    return launch_box_t<float>(v, d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
 }
 
 bool launch_box_shape_bf16(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout,
                            const uint16_t *wsrc, const uint16_t *vals, const uint16_t *g, uint16_t *out, float c2,
                            float mu, int clip, cudaStream_t st, cudaError_t *err)
 {
-    switch (v) {
-    case 1: return launch_box_var1_bf16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 2: return launch_box_var2_bf16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 3: return launch_box_var3_bf16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    default: return launch_box_var0_bf16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    }
+    using B = __nv_bfloat16;
+    return launch_box_t<B>(v, d, M, nx, ny, nz, np, p0, nout, reinterpret_cast<const B *>(wsrc),
+                           reinterpret_cast<const B *>(vals), reinterpret_cast<const B *>(g), reinterpret_cast<B *>(out),
+                           c2, mu, clip, st, err);
+}
+
+bool launch_box_shape_f16(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const __half *wsrc,
+                          const __half *vals, const __half *g, __half *out, float c2, float mu, int clip,
+                          cudaStream_t st, cudaError_t *err)
+{
+    return launch_box_t<__half>(v, d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
 }
 
 tnlm_status check_sweep_args(int nx, int ny, int nz, int np, int d, int M, float h, float mu)
@@ -294,40 +312,6 @@ tnlm_status launch_sweep(int nx, int ny, int nz, int np, const float *wsrc, cons
                          float *out, int d, int M, float h, float mu, int clip, cudaStream_t st)
 {
     return launch_sweep_range(nx, ny, nz, np, 0, np, wsrc, vals, g, out, d, M, h, mu, clip, st);
-}
-
-bool launch_box_grouped(int v, int d, int M, const GroupSweep *probs, int nprob, long long total,
-                        unsigned long long *counter, int sms, cudaStream_t st, cudaError_t *err)
-{
-    switch (v) {
-    case 1: return launch_box_grouped_var1(d, M, probs, nprob, total, counter, sms, st, err);
-    case 2: return launch_box_grouped_var2(d, M, probs, nprob, total, counter, sms, st, err);
-    case 3: return launch_box_grouped_var3(d, M, probs, nprob, total, counter, sms, st, err);
-    default: return launch_box_grouped_var0(d, M, probs, nprob, total, counter, sms, st, err);
-    }
-}
-
-bool box_grouped_tiles(int v, int d, int M, int nx, int ny, int nz, int np, int *ntx, int *nty, int *ntz,
-                       long long *items)
-{
-    switch (v) {
-    case 1: return box_grouped_tiles_var1(d, M, nx, ny, nz, np, ntx, nty, ntz, items);
-    case 2: return box_grouped_tiles_var2(d, M, nx, ny, nz, np, ntx, nty, ntz, items);
-    case 3: return box_grouped_tiles_var3(d, M, nx, ny, nz, np, ntx, nty, ntz, items);
-    default: return box_grouped_tiles_var0(d, M, nx, ny, nz, np, ntx, nty, ntz, items);
-    }
-}
-
-bool launch_box_shape_f16(int v, int d, int M, int nx, int ny, int nz, int np, int p0, int nout, const __half *wsrc,
-                          const __half *vals, const __half *g, __half *out, float c2, float mu, int clip,
-                          cudaStream_t st, cudaError_t *err)
-{
-    switch (v) {
-    case 1: return launch_box_var1_f16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 2: return launch_box_var2_f16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    case 3: return launch_box_var3_f16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    default: return launch_box_var0_f16(d, M, nx, ny, nz, np, p0, nout, wsrc, vals, g, out, c2, mu, clip, st, err);
-    }
 }
 
 tnlm_status launch_sweep_range_f16(int nx, int ny, int nz, int np, int p0, int nout, const __half *wsrc,
