@@ -16,7 +16,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtnlm.so")
 SOURCES = ["sweep_box_f32.cu", "sweep_box_f32b.cu", "sweep_box_bf16.cu", "sweep_box_f16.cu", "sweep_box_apart_f32.cu",
-           "sweep_box_apart_bf16.cu", "sweep_box_apart_f16.cu", "energy_box.cu", "projector.cu", "transpose.cu", "tnlm_sweep.cu",
+           "sweep_box_apart_bf16.cu", "sweep_box_apart_f16.cu", "energy_box.cu", "energy_box_bf16.cu",
+           "energy_box_f16.cu", "projector.cu", "transpose.cu", "tnlm_sweep.cu",
            "reduce.cu", "api.cu", "noalloc.cu", "cgls.cu", "fdk.cu", "energy.cu", "autotune.cu", "peaks.cu", "sweep_pairs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

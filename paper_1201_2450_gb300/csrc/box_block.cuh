@@ -91,6 +91,29 @@ __device__ __forceinline__ float2 xbox2(float2 b)
     }
 }
 
+// z box sums of BZ = 4 outputs from the differences t of their 4 + 2 D rows, the middle rows shared (sweep_tile.cuh).
+template <int D_, int BZ, int SZ, int SP>
+__device__ __forceinline__ void zsums(const float2 (&t)[SZ], float2 (&b)[BZ][SP], int p)
+{
+    static_assert(BZ == 4 && SZ == BZ + 2 * D_, "four outputs");
+    if constexpr (D_ == 1) {
+#pragma unroll
+        for (int k = 0; k < BZ; k += 2) {
+            const float2 m = __ffma2_rn(t[k + 2], t[k + 2], __fmul2_rn(t[k + 1], t[k + 1]));
+            b[k][p] = __ffma2_rn(t[k], t[k], m);
+            b[k + 1][p] = __ffma2_rn(t[k + 3], t[k + 3], m);
+        }
+    } else {
+        const float2 core = __ffma2_rn(t[4], t[4], __fmul2_rn(t[3], t[3]));
+        const float2 q1 = __ffma2_rn(t[1], t[1], __ffma2_rn(t[2], t[2], core));
+        const float2 q2 = __ffma2_rn(t[6], t[6], __ffma2_rn(t[5], t[5], core));
+        b[0][p] = __ffma2_rn(t[0], t[0], q1);
+        b[1][p] = __ffma2_rn(t[5], t[5], q1);
+        b[2][p] = __ffma2_rn(t[2], t[2], q2);
+        b[3][p] = __ffma2_rn(t[7], t[7], q2);
+    }
+}
+
 // Block shapes: (warps along y, warps along z, output rows per thread along z).
 template <int V> struct BoxShape;
 template <> struct BoxShape<0> { static constexpr int WY = 4, WZ = 2, BZ = 4; };  // 256 threads, tile 8 x 8
