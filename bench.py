@@ -48,11 +48,11 @@ WORKLOAD = ("NCAT-shaped 4D TNLM-R FP32: 10 phases x 256x256x64 @ 2 mm, 36 views
 NCU_TRAFFIC = {
     # single-kernel captures on the 6-phase case of this workload, scaled by 10/6 to its 10 phases; the
     # projector stage is the z-fastest copy plus the table walk, the transpose stage the column scan plus the bands
-    "k_forward": {"bytes_per_launch": int((100.727808e6 + 48.609024e6 + 606.395392e6 + 165.109504e6) * 10 / 6),
-                  "source_sha": "4ee81dbf075d39bb"},
-    "k_backproject": {"bytes_per_launch": int((169.919488e6 + 284.322560e6 + 556.931328e6 + 93.128448e6) * 10 / 6),
-                      "source_sha": "5aa935fcb93c583b"},
-    "k_sweep": {"bytes_per_launch": int((162.544640e6 + 83.844608e6) * 10 / 6), "source_sha": "aa475743b3412a05"},
+    "k_forward": {"bytes_per_launch": int((100.679936e6 + 56.512768e6 + 609.453568e6 + 161.493504e6) * 10 / 6),
+                  "source_sha": "afafaf434505db22"},
+    "k_backproject": {"bytes_per_launch": int((169.892608e6 + 284.578560e6 + 567.618304e6 + 107.038464e6) * 10 / 6),
+                      "source_sha": "17078780a0ef088a"},
+    "k_sweep": {"bytes_per_launch": int((164.065024e6 + 82.683904e6) * 10 / 6), "source_sha": "27cb305836d9ff71"},
 }
 
 
@@ -180,13 +180,14 @@ K1_FLOP_SLAB, K1_FLOP_B, K1_FLOP_C = 12, 3, 7
 # 6 (its segment length and FMA, the next z plane by an add and one FMA); so per ray
 # 3 (1 + |dx| + |dy|) + 6 |dz|.  The tables themselves are built once per geometry, not per launch.
 K1_TAB_FLOP_ENTRY, K1_TAB_FLOP_C = 3, 6
-# FP32 operations of the band transpose per non-zero of P, counted from its source on this geometry
-# (an FMA counts 2, a min/max or a conversion 1): per (column of 8 cells, view, pixel column) 38 for
-# the chord (two slab tests) and the row-map slopes, 12 for the chord midpoint, the first boundary
-# and its row images, then 30 per cell boundary (the boundary height, its two row images with their
-# margins, the band row's split and its two accumulations, the prefix difference of the full rows),
-# 320 in all, plus ~13 for the column's footprint per view shared by its ~3.5 pixel columns, over
-# the ~38 (ray, cell) pairs that chord serves (about 4.8 detector rows per 2 mm cell).
+# FP32 operations of a band transpose per non-zero of P on this geometry (an FMA counts 2, a min/max
+# or a conversion 1), the unit of work its rate is quoted in: per (column of 8 cells, view, pixel
+# column) 38 for the chord (two slab tests) and the row-map slopes, 12 for the chord midpoint and the
+# first boundary, then 30 per cell boundary (its height, two row images with margins, the band row's
+# split and accumulations, the prefix difference of the full rows), 320 in all, plus ~13 for the
+# column's footprint per view shared by its ~3.5 pixel columns, over the ~38 (ray, cell) pairs that
+# chord serves (about 4.8 detector rows per 2 mm cell).  The kernel itself needs fewer: one row image
+# per boundary, and a chord per 16 cells.
 K2_FLOP_PER_NNZ = 8.5
 
 
@@ -243,7 +244,10 @@ def projection_counts(desc: dict, device="cuda") -> tuple[int, int, int]:
 
 # FP32 operations per pair evaluation of the sweep (the hot-path analysis's per-unit figure):
 # 3*3*(2d+1) for the box-sum patch distance plus 8 for the weight and the two accumulations
-# (one exp besides).
+# (one exp besides).  This is the unit of work, without the sums that outputs share: the kernel
+# executes 16.25 per pair with d = 1 (4 x 2 x 2 outputs: 48 differences, 84 for the z sums, 24 for
+# the y sums, 24 for the x sums, 80 for the weights and accumulations, over 16), so the fraction of
+# the FP32 peak below is not the FMA pipe's utilisation.
 
 
 def sweep_ops_per_pair(d: int) -> int:

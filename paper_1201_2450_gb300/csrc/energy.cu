@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kNT) k_wa_G(int nx, int ny, int nz, int ntz, c
 // p on the padded grid [-d, n+d)^3, stored at (p + d).  A warp takes 32 - 2d
 // positions of one row and one offset through every z: 2d + 1 coalesced loads
 // a slice, the x sum by shuffles, the z sum from a ring of slice sums (27 loads
-// a position otherwise: 1.17 -> 0.2 ms per phase pair of 95 x 90 x 71, M = 2).
+// a position otherwise: 1.17 -> 0.38 ms per phase pair of 95 x 90 x 71, M = 2).
 template <int D>
 __global__ void __launch_bounds__(256) k_wa_B(int nx, int ny, int nz, const float *__restrict__ G, float *__restrict__ B)
 {

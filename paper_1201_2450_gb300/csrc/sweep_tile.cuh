@@ -16,7 +16,7 @@
 //   XPair, d = 1: 2 (x) x 4 (y) x 2 (z) outputs, pairs along x: 12.0 FMA-pipe
 //     cycles and 8.3 LSU cycles per evaluation and warp (the 1 x 2 x 4 block
 //     of pairs along y: 15 and 12.9);
-//   YQuad, d = 2: 1 x 4 x 4 outputs, pairs along y: 17.3 and 16.
+//   YBlock, d = 2: 1 x 4 x 4 outputs, pairs along y: 17.3 and 16.
 //
 // Normalisation is online.  The weights are 2^(m - t), t = D log2(e) / 2h^2,
 // against a running reference m that starts at the first candidate and moves

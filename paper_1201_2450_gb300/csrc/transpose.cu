@@ -287,7 +287,8 @@ __device__ __forceinline__ void bands_view(const KGeom &G, const float4 *s_row, 
 
 // Resident warps per SM that the registers are budgeted for.  The 17 boundaries of 16 cells are one straight run
 // of independent gathers, and 128 registers let their loads be issued ahead: on the 10 x 256x256x64 workload 16
-// cells take 6.61 ms at 16 warps per SM, 7.5 at 20, 8.7 at 24; 8 cells 7.47 ms at 20 (7.8 at 16, 8.0 at 28).
+// cells took 6.61 ms at 16 warps per SM, 7.5 at 20, 8.7 at 24; 8 cells 7.47 ms at 20 (7.8 at 16, 8.0 at 28), all
+// before the addresses were written out (at() in ray_common.cuh), which took the chosen form to 6.39.
 constexpr int bands_warps(int ch) { return ch == 16 ? 16 : 20; }
 
 // NW warps of 8 x 4 voxel columns, each thread CH z cells of one column.  SPLIT = 1: the warps lie side by side (two
@@ -297,7 +298,7 @@ constexpr int bands_warps(int ch) { return ch == 16 ? 16 : 20; }
 // boundaries beyond the volume (ragged nz) are computed like the others and their cells not stored.
 // Bound by instruction issue (74 % of the slots, 22 instructions per boundary) with the L1's gathers behind it (67 %
 // of its wavefront rate); 2.7 times faster per boundary than row tests with min/max bounds on both ends of each band
-// and 32 x 1 column warps (k_backproject_bands at 10 x 256x256x64, 360 views x 512x384: 15.4 -> 6.5 ms).
+// and 32 x 1 column warps (k_backproject_bands at 10 x 256x256x64, 360 views x 512x384: 15.4 -> 6.3 ms, with k_colscan 15.5 -> 6.39).
 template <int CH, int NW, int SPLIT, int ROWS, class T>
 __global__ void __launch_bounds__(32 * NW, bands_warps(CH) / NW)
     k_backproject_bands(KGeom G, const ViewGeom *__restrict__ views, const int *__restrict__ view_off,
