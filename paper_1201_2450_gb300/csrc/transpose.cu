@@ -291,21 +291,22 @@ __device__ __forceinline__ void bands_view(const KGeom &G, const float4 *s_row, 
 // before the addresses were written out (at() in ray_common.cuh), which took the chosen form to 6.39.
 constexpr int bands_warps(int ch) { return ch == 16 ? 16 : 20; }
 
-// NW warps of 8 x 4 voxel columns, each thread CH z cells of one column.  SPLIT = 1: the warps lie side by side (two
-// along x) and each sums every view of the phase.  SPLIT = NW: the warps share one patch of columns, warp w takes the
-// views w, w + NW, ... and the partial sums are added in warp order: for volumes too small to fill the GPU otherwise.
+// NW warps of 8 x 4 voxel columns, each thread CH z cells of one column.  A voxel is the sum of ORDER partial sums over
+// the views p, p + ORDER, ... of its phase, p = 0, 1, ... added in that order.  SPLIT = 1: the warps lie side by side
+// (two along x) and each takes every partial sum in turn (those before in shared memory).  SPLIT = ORDER = NW: the warps
+// share one patch of columns and warp p takes partial sum p, for launches too small to fill the GPU otherwise.
 // The input is the ray-length-scaled residual (k_colscan writes a scaled copy of an unscaled input).  The chunk's
 // boundaries beyond the volume (ragged nz) are computed like the others and their cells not stored.
 // Bound by instruction issue (74 % of the slots, 22 instructions per boundary) with the L1's gathers behind it (67 %
 // of its wavefront rate); 2.7 times faster per boundary than row tests with min/max bounds on both ends of each band
 // and 32 x 1 column warps (k_backproject_bands at 10 x 256x256x64, 360 views x 512x384: 15.4 -> 6.3 ms, with k_colscan 15.5 -> 6.39).
-template <int CH, int NW, int SPLIT, int ROWS, class T>
+template <int CH, int NW, int SPLIT, int ORDER, int ROWS, class T>
 __global__ void __launch_bounds__(32 * NW, bands_warps(CH) / NW)
     k_backproject_bands(KGeom G, const ViewGeom *__restrict__ views, const int *__restrict__ view_off,
                         const float *__restrict__ proj, const float2 *__restrict__ pref, const T *vin,
                         T *vout, float alpha, float beta, int nchunks)
 {
-    static_assert(SPLIT == 1 || SPLIT == NW, "warps lie side by side or share one patch");
+    static_assert(SPLIT == 1 || (SPLIT == NW && SPLIT == ORDER), "warps lie side by side or share one patch");
     constexpr int NT = 32 * NW;
     extern __shared__ float4 sm4[];
     float4 *s_row = sm4;  // per detector row: (v, 1/|v| or +inf, sign of v (+1 for v = 0), 0); [nv], [nv + 1]: no row
@@ -327,16 +328,33 @@ __global__ void __launch_bounds__(32 * NW, bands_warps(CH) / NW)
     float acc[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k) acc[k] = 0.f;
+    float *s_acc = reinterpret_cast<float *>(s_row + G.nv + 2);  // partial sums: [NW - 1][CH][32], unsplit [CH][NT]
     if (inside) {
         const float xc = G.b0x + ((float)ix + 0.5f) * G.dx;
         const float yc = G.b0y + ((float)iy + 0.5f) * G.dy;
-        const int v_end = view_off[phase + 1];
-        for (int vg = view_off[phase] + (SPLIT > 1 ? warp : 0); vg < v_end; vg += SPLIT)
-            bands_view<CH, ROWS>(G, s_row, views[vg].c, views[vg].s, xc, yc, iz0, proj + (long long)vg * G.npix,
-                                  pref + (long long)vg * (G.nv + 1) * G.nu, acc);
+        const int v0 = view_off[phase], v_end = view_off[phase + 1];
+        auto add_views = [&](int first) {
+            for (int vg = v0 + first; vg < v_end; vg += ORDER)
+                bands_view<CH, ROWS>(G, s_row, views[vg].c, views[vg].s, xc, yc, iz0, proj + (long long)vg * G.npix,
+                                      pref + (long long)vg * (G.nv + 1) * G.nu, acc);
+        };
+        if (SPLIT > 1 || ORDER == 1) {
+            add_views(SPLIT > 1 ? warp : 0);
+        } else {
+            for (int p = 0; p < ORDER; ++p) {  // a thread reads only what it wrote itself
+                add_views(p);
+#pragma unroll
+                for (int k = 0; k < CH; ++k) {
+                    if (p > 0) acc[k] = s_acc[k * NT + tid] + acc[k];
+                    if (p < ORDER - 1) {
+                        s_acc[k * NT + tid] = acc[k];
+                        acc[k] = 0.f;
+                    }
+                }
+            }
+        }
     }
     if (SPLIT > 1) {
-        float *s_acc = reinterpret_cast<float *>(s_row + G.nv + 2);  // [NW - 1][CH][32]
         if (warp > 0)
 #pragma unroll
             for (int k = 0; k < CH; ++k) s_acc[((warp - 1) * CH + k) * 32 + lane] = acc[k];
@@ -395,15 +413,16 @@ static int band_rows(const KGeom &kg)
     return rows <= 0.98 ? 1 : (rows <= 1.98 ? 2 : 0);
 }
 
-template <int CH, int NW, int SPLIT, int ROWS, class T>
+template <int CH, int NW, int SPLIT, int ORDER, int ROWS, class T>
 static tnlm_status launch_bands_m(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                   const float2 *pref, const T *vin, T *vout, float alpha, float beta, cudaStream_t st)
 {
     const int nchb = (kg.nz + CH - 1) / CH;
     constexpr int TX = SPLIT > 1 ? kBandWX : 2 * kBandWX, TY = SPLIT > 1 ? kBandWY : (NW / 2) * kBandWY;
     dim3 grid((kg.nx + TX - 1) / TX, (kg.ny + TY - 1) / TY, kg.np * nchb);
-    const size_t smem = sizeof(float4) * (kg.nv + 2) + (SPLIT > 1 ? sizeof(float) * (NW - 1) * CH * 32 : 0);
-    auto kern = k_backproject_bands<CH, NW, SPLIT, ROWS, T>;
+    const size_t smem = sizeof(float4) * (kg.nv + 2) +
+                        sizeof(float) * CH * (SPLIT > 1 ? (NW - 1) * 32 : (ORDER > 1 ? NW * 32 : 0));
+    auto kern = k_backproject_bands<CH, NW, SPLIT, ORDER, ROWS, T>;
     if (smem > 48 * 1024)
         TNLM_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<grid, 32 * NW, smem, st>>>(kg, views, view_off, src, pref, vin, vout, alpha, beta, nchb);
@@ -413,51 +432,62 @@ static tnlm_status launch_bands_m(const KGeom &kg, const ViewGeom *views, const 
 
 // Wide bands run in one shape per form (the result does not depend on it): pixels that fine against the voxels are
 // rare, and the row loop, not the shape, sets their time.
-template <int CH, int NW, int SPLIT, class T>
+template <int CH, int NW, int SPLIT, int ORDER, class T>
 static tnlm_status launch_bands(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                 const float2 *pref, const T *vin, T *vout, float alpha, float beta, cudaStream_t st)
 {
     switch (band_rows(kg)) {
-    case 1: return launch_bands_m<CH, NW, SPLIT, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    case 2: return launch_bands_m<CH, NW, SPLIT, 2, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    default: return launch_bands_m<8, 4, SPLIT, 0, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    case 1: return launch_bands_m<CH, NW, SPLIT, ORDER, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    case 2: return launch_bands_m<CH, NW, SPLIT, ORDER, 2, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    default: return launch_bands_m<8, 4, SPLIT, ORDER, 0, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     }
 }
 
-// Blocks of 16 x 8 voxel columns and ch cells
-static long long band_blocks(const KGeom &kg, int ch)
+// Blocks of 16 x 8 voxel columns and ch cells that np phases make
+static long long band_blocks(const KGeom &kg, int np, int ch)
 {
-    return (long long)((kg.nx + 15) / 16) * ((kg.ny + 7) / 8) * kg.np * ((kg.nz + ch - 1) / ch);
+    return (long long)((kg.nx + 15) / 16) * ((kg.ny + 7) / 8) * np * ((kg.nz + ch - 1) / ch);
 }
 
-// The form of the band transpose by size.  A launch fills the GPU from about one block per resident slot (152 SMs x 4
-// blocks).  Below that, with chunks of 8 cells, the four warps of a block split the views of one patch instead (4 x
-// 32^3, 20 views: stage 37 -> 25 us; 27 us in chunks of 4); the split depends on the geometry alone, so every launch
-// shape sums in the same order.  With bp_ch = 8 and bp_by = 4 (the defaults) the chunk is 16 cells where the volume has
-// them: a thread's chord set-up serves twice the cells (6.61 against 7.47 ms at 10 x 256x256x64), which padding an
-// odd number of 8-cell chunks must not eat up.
+// A launch fills the GPU from about this many blocks: four resident on each of the 152 SMs.
 constexpr long long kBandsFill = 152 * 4;
 
+// The forms of the order of summation ORDER, by size.  With bp_ch = 8 and bp_by = 4 (the defaults) the chunk is 16 cells
+// where the volume has them: a thread's chord set-up serves twice the cells (6.61 against 7.47 ms at 10 x 256x256x64),
+// which padding an odd number of 8-cell chunks must not eat up.
+template <int ORDER, class T>
+static tnlm_status launch_bands_shape(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
+                                      const float2 *pref, const T *vin, T *vout, float alpha, float beta,
+                                      cudaStream_t st)
+{
+    const int n8 = (kg.nz + 7) / 8;
+    if (kg.bp_ch == 8 && kg.bp_by == 4 && band_blocks(kg, kg.np, 16) >= kBandsFill && (n8 % 2 == 0 || n8 > 8))
+        return launch_bands<16, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 8 && kg.bp_by == 4)
+        return launch_bands<8, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 8 && kg.bp_by == 2)
+        return launch_bands<8, 2, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 4 && kg.bp_by == 4)
+        return launch_bands<4, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    return launch_bands<4, 2, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+}
+
+// The form of the band transpose by size.  Volumes of which one phase does not fill the GPU are summed in four partial
+// sums, so that the warps of a block can split the views of one patch where the whole launch does not fill it either
+// (4 x 32^3, 20 views: stage 37 -> 25 us; 27 us in chunks of 4).  The order depends on the volume alone, not on how many
+// phases the handle holds, so a rank that holds some of a scan's phases gets the bits of a process that holds all.
 template <class T>
 static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                         const float2 *pref, const T *vin, T *vout, float alpha, float beta,
                                         cudaStream_t st)
 {
-    if (band_blocks(kg, 8) < kBandsFill) {
-        if (kg.bp_ch == 8)
-            return launch_bands<8, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-        return launch_bands<4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    }
-    const int n8 = (kg.nz + 7) / 8;
-    if (kg.bp_ch == 8 && kg.bp_by == 4 && band_blocks(kg, 16) >= kBandsFill && (n8 % 2 == 0 || n8 > 8))
-        return launch_bands<16, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 8 && kg.bp_by == 4)
-        return launch_bands<8, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 8 && kg.bp_by == 2)
-        return launch_bands<8, 2, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 4 && kg.bp_by == 4)
-        return launch_bands<4, 4, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    return launch_bands<4, 2, 1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (band_blocks(kg, 1, 8) >= kBandsFill)
+        return launch_bands_shape<1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (band_blocks(kg, kg.np, 8) >= kBandsFill)
+        return launch_bands_shape<4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    if (kg.bp_ch == 8)
+        return launch_bands<8, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
+    return launch_bands<4, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
 }
 
 template <class T>
