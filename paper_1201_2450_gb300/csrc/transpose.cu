@@ -452,6 +452,11 @@ static long long band_blocks(const KGeom &kg, int np, int ch)
 // A launch fills the GPU from about this many blocks: four resident on each of the 152 SMs.
 constexpr long long kBandsFill = 152 * 4;
 
+// Cells per thread: chunks of 8 where bp_ch asks for them and the volume has more than 4 slices, as the boundaries
+// beyond the volume cost what the others do (6 x 192x192x1, 30 views of 256x192: 290 us in chunks of 8, 225 of 4; one
+// phase of 256x256x1, 360 views of 512x64: 985 and 665).
+static int band_cells(const KGeom &kg) { return kg.nz <= 4 ? 4 : kg.bp_ch; }
+
 // The forms of the order of summation ORDER, by size.  With bp_ch = 8 and bp_by = 4 (the defaults) the chunk is 16 cells
 // where the volume has them: a thread's chord set-up serves twice the cells (6.61 against 7.47 ms at 10 x 256x256x64),
 // which padding an odd number of 8-cell chunks must not eat up.
@@ -460,14 +465,14 @@ static tnlm_status launch_bands_shape(const KGeom &kg, const ViewGeom *views, co
                                       const float2 *pref, const T *vin, T *vout, float alpha, float beta,
                                       cudaStream_t st)
 {
-    const int n8 = (kg.nz + 7) / 8;
-    if (kg.bp_ch == 8 && kg.bp_by == 4 && band_blocks(kg, kg.np, 16) >= kBandsFill && (n8 % 2 == 0 || n8 > 8))
+    const int n8 = (kg.nz + 7) / 8, ch = band_cells(kg);
+    if (ch == 8 && kg.bp_by == 4 && band_blocks(kg, kg.np, 16) >= kBandsFill && (n8 % 2 == 0 || n8 > 8))
         return launch_bands<16, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 8 && kg.bp_by == 4)
+    if (ch == 8 && kg.bp_by == 4)
         return launch_bands<8, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 8 && kg.bp_by == 2)
+    if (ch == 8 && kg.bp_by == 2)
         return launch_bands<8, 2, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 4 && kg.bp_by == 4)
+    if (ch == 4 && kg.bp_by == 4)
         return launch_bands<4, 4, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     return launch_bands<4, 2, 1, ORDER, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
 }
@@ -485,7 +490,7 @@ static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, 
         return launch_bands_shape<1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     if (band_blocks(kg, kg.np, 8) >= kBandsFill)
         return launch_bands_shape<4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (kg.bp_ch == 8)
+    if (band_cells(kg) == 8)
         return launch_bands<8, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     return launch_bands<4, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
 }

@@ -1,0 +1,42 @@
+"""Small and thin problems cost less than the ones whose launches they share:
+each test compares a call with one that does several times its work.  Minima
+of repeated runs; the limits leave a third of the measured difference as room."""
+import pytest
+import torch
+
+import paper_1201_2450_gb300 as tnlm
+from paper_1201_2450_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def time_us(fn, repeats=7, calls=10):
+    fn()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(repeats):
+        a.record()
+        for _ in range(calls):
+            fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / calls * 1e3)
+    return best
+
+
+def scan(nx, ny, nz, nu, nv, views, **kw):
+    d = dict(dx=2.0, du=1.56, sad=1000.0, sdd=1500.0, angle_offset=0.07)
+    d.update(kw)
+    return tnlm.Geometry(synth.make_geometry(nx=nx, ny=ny, nz=nz, nu=nu, nv=nv, n_phases=len(views),
+                                             views_per_phase=views, **d))
+
+
+def backproject_us(G):
+    y, v = torch.rand(G.proj_shape, device="cuda"), torch.empty(G.vol_shape, device="cuda")
+    return time_us(lambda: tnlm.tnlm_backproject(G, y, v))
+
+
+def test_transpose_of_one_slice():
+    """One slice against eight: measured 0.68 (1.0 when both took chunks of 8)."""
+    one, eight = (backproject_us(scan(256, 256, nz, 512, 64, [180], du=0.78)) for nz in (1, 8))
+    assert one < 0.85 * eight
