@@ -449,8 +449,9 @@ static long long band_blocks(const KGeom &kg, int np, int ch)
     return (long long)((kg.nx + 15) / 16) * ((kg.ny + 7) / 8) * np * ((kg.nz + ch - 1) / ch);
 }
 
-// A launch fills the GPU from about this many blocks: four resident on each of the 152 SMs.
-constexpr long long kBandsFill = 152 * 4;
+// A launch fills the GPU from about kBandsFill blocks, four resident on each of the 152 SMs; kBandsSplit is where the
+// launches that take their partial sums in turn become the faster ones.
+constexpr long long kBandsFill = 152 * 4, kBandsSplit = 152 * 10;
 
 // Cells per thread: chunks of 8 where bp_ch asks for them and the volume has more than 4 slices, as the boundaries
 // beyond the volume cost what the others do (6 x 192x192x1, 30 views of 256x192: 290 us in chunks of 8, 225 of 4; one
@@ -478,9 +479,11 @@ static tnlm_status launch_bands_shape(const KGeom &kg, const ViewGeom *views, co
 }
 
 // The form of the band transpose by size.  Volumes of which one phase does not fill the GPU are summed in four partial
-// sums, so that the warps of a block can split the views of one patch where the whole launch does not fill it either
-// (4 x 32^3, 20 views: stage 37 -> 25 us; 27 us in chunks of 4).  The order depends on the volume alone, not on how many
-// phases the handle holds, so a rank that holds some of a scan's phases gets the bits of a process that holds all.
+// sums, so that the warps of a block can split the views of one patch where the whole launch is small (4 x 32^3, 20
+// views: stage 37 -> 25 us; 27 us in chunks of 4).  The order depends on the volume alone, not on how many phases the
+// handle holds, so a rank that holds some of a scan's phases gets the bits of a process that holds all.  Partial sums in
+// turn / split, 36 views a phase, by the launch's blocks: 768 (6 of 64x64x32) 175 / 142 us, 1024 (4 of 64^3) 197 / 186,
+// 1280 (10 of 64x64x32) 241 / 219, 1536 (6 of 64^3) 267 / 265, 2304 (4 of 96x96x64) 343 / 378, 2560 (10 of 64^3) 416 / 446.
 template <class T>
 static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                         const float2 *pref, const T *vin, T *vout, float alpha, float beta,
@@ -488,7 +491,7 @@ static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, 
 {
     if (band_blocks(kg, 1, 8) >= kBandsFill)
         return launch_bands_shape<1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (band_blocks(kg, kg.np, 8) >= kBandsFill)
+    if (band_blocks(kg, kg.np, 8) >= kBandsSplit)
         return launch_bands_shape<4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     if (band_cells(kg) == 8)
         return launch_bands<8, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
