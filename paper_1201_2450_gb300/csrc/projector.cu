@@ -427,7 +427,8 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
             Ez[j] = (G.alpha0 * v - G.b0z) * G.inv_dz;
             Gz[j] = v * G.inv_dz;
             const float za = fmaf(blo, Gz[j], Ez[j]), zb = fmaf(bhi, Gz[j], Ez[j]);
-            const float margin = fmaf(fabsf(Gz[j]), 1e-6f, 1e-3f);
+            // at the top face z is known to half an ulp of nz, more than the 1e-3 beyond 2^14 slices
+            const float margin = fmaf(fabsf(Gz[j]), 1e-6f, fmaxf(1e-3f, fnz * 0x1p-22f));
             if (fminf(za, zb) >= margin && fmaxf(za, zb) <= fnz - margin) {
                 lo = blo;
                 hi = bhi;
