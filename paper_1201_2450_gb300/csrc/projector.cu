@@ -376,6 +376,32 @@ __device__ __forceinline__ float add_planes(const float4 *__restrict__ head, con
     return sum;
 }
 
+// The walk of one row with every entry split at its z planes in turn, for a row whose sum is not finite: the differences
+// of add_planes make NaN of an infinite voxel next to a plane (inf - inf).  A voxel that the row has no part in is not
+// read.
+__device__ __noinline__ float walk_row(const float4 *__restrict__ head, const float4 &h1, const float *__restrict__ fp,
+                                       int nz, float ez, float gz)
+{
+    const float2 *__restrict__ tc = reinterpret_cast<const float2 *>(head) + kColtabHead;
+    const int K = __float_as_int(h1.x), step = gz > 0.f ? 1 : -1;
+    const float iv = gz != 0.f ? 1.0f / gz : 0.f, ov = -ez * iv, fnz = (float)nz;
+    auto cell = [&](float e) { return (int)floorf(fminf(fmaxf(fmaf(e, gz, ez), -1.f), fnz)); };
+    float sum = 0.f, cur = h1.z;
+    int i = cell(cur);
+    for (int k = 0; k < K; ++k) {
+        const float2 t = __ldg(tc + k);
+        const int last = cell(t.x);
+        for (int n = max((last - i) * step, 0); n >= 0; --n, i += step) {  // n planes left in the entry
+            const float plane = (float)(i + (step > 0 ? 1 : 0));
+            const float end = n > 0 ? fminf(fmaxf(fmaf(plane, iv, ov), cur), t.x) : t.x;
+            if (end > cur && i >= 0 && i < nz) sum = fmaf(__ldg(fp + (__float_as_int(t.y) + i)), end - cur, sum);
+            cur = end;
+        }
+        i = last;
+    }
+    return sum;
+}
+
 // A warp walks 32 R rows of one detector column (block: NC adjacent columns), R per lane, 32 apart.
 // Along an entry's segment e_{k-1} .. e_k a row stays in one voxel unless it crosses a z plane there, once in ~25
 // entries.  The walk takes every entry whole, with the voxel at its end:
@@ -549,9 +575,12 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
         const float4 *__restrict__ head =
             reinterpret_cast<const float4 *>(G.coltab + coltab_base(vg, iu, G.coltab_kmax, G.nu));
         const float4 h1 = __ldg(head + 1);
-        if (__float_as_int(h1.x) > 0)
-            sum = add_planes(head, h1, vol + (long long)V.phase * G.nvox, G.nz, (G.alpha0 * v - G.b0z) * G.inv_dz,
-                             v * G.inv_dz, sum);
+        if (__float_as_int(h1.x) > 0) {
+            const float *__restrict__ fp = vol + (long long)V.phase * G.nvox;
+            const float ez = (G.alpha0 * v - G.b0z) * G.inv_dz, gz = v * G.inv_dz;
+            sum = add_planes(head, h1, fp, G.nz, ez, gz, sum);
+            if (!(fabsf(sum) <= FLT_MAX)) sum = walk_row(head, h1, fp, G.nz, ez, gz);
+        }
         const float Dx = -G.sdd * V.c - u * V.s, Dy = -G.sdd * V.s + u * V.c;
         const float len = sqrtf(Dx * Dx + Dy * Dy + v * v);
         const float pf = sum * len;
