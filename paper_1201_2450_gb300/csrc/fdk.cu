@@ -51,6 +51,14 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
         const float u = ((float)i - G.uc) * G.du + G.u_off;
         return __ldg(pr + (long long)r * G.nu + i) * G.sdd * rsqrtf(s_q[r] + u * u);
     };
+    // The far taps of one output, in the tiles' order, where the tiles' sum is not finite: their zeros for the near taps
+    // make NaN of an infinite sample (0 * inf) that only the near sum holds.
+    auto far_taps = [&](int r, int n) {
+        float sum = 0.f;
+        for (int i = 1 - p; i < G.nu; i += 2)
+            if (abs(n - i) > kNear) sum = fmaf(weighted(r, i), hs / ((float)(n - i) * (float)(n - i)), sum);
+        return sum;
+    };
     float acc[8][8];  // [row][output]
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -117,7 +125,9 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
             float near = h0 * c[0];
 #pragma unroll
             for (int m = 1; m <= kNear; m += 2) near = fmaf(hs / (float)(m * m), c[-m] + c[m], near);
-            if (n < G.nu) filt[row * G.nu + n] = G.du * (near + s_o[o]);
+            float far = s_o[o];
+            if (!(fabsf(far) <= FLT_MAX)) far = far_taps(8 * warp + r, n);
+            if (n < G.nu) filt[row * G.nu + n] = G.du * (near + far);
         }
     }
 }
