@@ -30,6 +30,18 @@ constexpr int kFiltPitch = kFiltRows + 4;
 constexpr int kNear = 15;                                // odd
 constexpr int kFiltStrip = 2 * kFiltOut + 2 * kNear + 2;  // samples around a block's outputs in one row
 
+// The far taps of output n of one row, in the tiles' order, where the tiles' sum is not finite: their zeros for the near
+// taps make NaN of an infinite sample (0 * inf) that only the near sum holds.  q: SDD^2 + v^2 of the row.
+__device__ __noinline__ float far_taps(const KGeom &G, const float *__restrict__ row, float q, float hs, int n)
+{
+    float sum = 0.f;
+    for (int i = (n + 1) & 1; i < G.nu; i += 2) {
+        const float u = ((float)i - G.uc) * G.du + G.u_off, m = (float)(n - i);
+        if (abs(n - i) > kNear) sum = fmaf(__ldg(row + i) * G.sdd * rsqrtf(q + u * u), hs / (m * m), sum);
+    }
+    return sum;
+}
+
 __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long long rows, const float *__restrict__ proj,
                                                                 float *__restrict__ filt)
 {
@@ -50,14 +62,6 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
     auto weighted = [&](int r, int i) {  // R' at sample i of the block's row r
         const float u = ((float)i - G.uc) * G.du + G.u_off;
         return __ldg(pr + (long long)r * G.nu + i) * G.sdd * rsqrtf(s_q[r] + u * u);
-    };
-    // The far taps of one output, in the tiles' order, where the tiles' sum is not finite: their zeros for the near taps
-    // make NaN of an infinite sample (0 * inf) that only the near sum holds.
-    auto far_taps = [&](int r, int n) {
-        float sum = 0.f;
-        for (int i = 1 - p; i < G.nu; i += 2)
-            if (abs(n - i) > kNear) sum = fmaf(weighted(r, i), hs / ((float)(n - i) * (float)(n - i)), sum);
-        return sum;
     };
     float acc[8][8];  // [row][output]
 #pragma unroll
@@ -126,7 +130,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
 #pragma unroll
             for (int m = 1; m <= kNear; m += 2) near = fmaf(hs / (float)(m * m), c[-m] + c[m], near);
             float far = s_o[o];
-            if (!(fabsf(far) <= FLT_MAX)) far = far_taps(8 * warp + r, n);
+            if (!(fabsf(far) <= FLT_MAX)) far = far_taps(G, proj + row * G.nu, s_q[8 * warp + r], hs, n);
             if (n < G.nu) filt[row * G.nu + n] = G.du * (near + far);
         }
     }
