@@ -164,11 +164,14 @@ __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restr
         const float u = G.sdd * (-x * s + y * c) * iU;
         const float fu = (u - G.u_off) * G.inv_du + G.uc;
         const float fu0 = floorf(fu);
-        if (!(fu0 >= -1.f && fu0 < (float)G.nu)) continue;  // both columns off the detector
+        if (!(fu > -1.f && fu < (float)G.nu)) continue;  // both columns off the detector
         const int iu0 = (int)fu0;
         const float au = fu - fu0, wv = wscale * iU * iU;
-        // a column off the detector reads its neighbour with weight 0
-        const float wb = iu0 + 1 < G.nu ? au : 0.f, wa = iu0 >= 0 ? 1.f - au : 0.f;
+        // a column off the detector reads its neighbour, at half that one's weight each (with weight 0 an infinite
+        // neighbour would make NaN; a select per gather took the call at 10 x 256x256x64 from 2.89 to 3.80 ms)
+        const bool in_a = iu0 >= 0, in_b = iu0 + 1 < G.nu;
+        const float wa = in_a ? (in_b ? 1.f : 0.5f) * (1.f - au) : 0.5f * au;
+        const float wb = in_a && in_b ? au : wa;
         const int ca = max(iu0, 0), cb = min(iu0 + 1, G.nu - 1);
         const float *__restrict__ F = filt + (long long)vg * G.npix;
         const float *__restrict__ Fa = F + ca, *__restrict__ Fb = F + cb;

@@ -2,8 +2,9 @@
 has a positive tap at 0, negative taps at odd offsets and none at even ones, so
 the filtered row is +inf at the pixel, -inf at the columns of the other parity
 and finite elsewhere; a voxel takes two neighbouring columns, one of each
-parity, and is -inf wherever neither is the pixel itself: far from it
-and near it (the taps that are summed apart)."""
+parity, and is -inf wherever neither is the pixel itself: far from it, near
+it (the taps that are summed apart), and where one of the two columns lies off
+the detector and the voxel takes only the other."""
 import numpy as np
 import pytest
 import torch
@@ -27,7 +28,7 @@ def images(desc):
     return np.broadcast_to(fu, fv.shape), fv
 
 
-@pytest.mark.parametrize("where", ["near", "far"])
+@pytest.mark.parametrize("where", ["near", "far", "left_edge", "right_edge"])
 @pytest.mark.parametrize("column", [31, 33])
 def test_infinite_pixel(column, where):
     desc = synth.make_geometry(nx=70, ny=66, nz=14, dx=1.0, nu=NU, nv=NV, du=1.2, dv=1.2, sad=300.0, sdd=450.0, n_phases=1,
@@ -40,7 +41,8 @@ def test_infinite_pixel(column, where):
     rows = np.abs(fv - ROW) < 0.999  # the infinite row has a share
     clear = np.abs(fv - ROW) > 1.001
     away = np.abs(fu - column)
-    sel = {"near": (away > 1.001) & (away < 14) & (fu > 0.001), "far": (away > 16) & (fu > 0.001) & (fu < NU - 1.001)}[where]
+    sel = {"near": (away > 1.001) & (away < 14) & (fu > 0.001), "far": (away > 16) & (fu > 0.001) & (fu < NU - 1.001),
+           "left_edge": (fu > -0.999) & (fu < -0.001), "right_edge": (fu > NU - 0.999) & (fu < NU - 0.001)}[where]
     assert (sel & rows).sum() > 20
     assert np.isneginf(vol[sel & rows]).all()
     assert np.isfinite(vol[clear]).all()
