@@ -18,17 +18,37 @@ namespace {
 // The ramp's even taps vanish apart from h[0], so the outputs of one parity are a dense convolution of the samples of
 // the other:  F(u_{2j+p}) = du (h[0] R'_{2j+p} + sum_k h[2(j - k) + 2p - 1] R'_{2k+1-p}).
 // A block takes 64 detector rows and 256 outputs of one parity: per sample k a thread multiplies 8 rows (one 32-byte
-// broadcast) by 8 consecutive outputs' taps, which slide through registers (two 16-byte loads per four samples), so
-// the FMA pipe binds (64 FMAs to 10 shared-memory cycles a sample and warp).  138 k rows of 512: 5.7 -> 1.3 ms against
-// one output per thread with three shared loads to two taps.
+// broadcast) by 8 consecutive outputs' taps, which slide through registers (two 16-byte loads per four samples).  138 k
+// rows of 512: 5.7 -> 1.33 ms against one output per thread with three shared loads to two taps, 36 % of the FMA peak by
+// operations; the chunks' loads and barriers are not overlapped with the products.  Short rows and few rows take a tile of
+// 16 x 64 (filter_small), which sums every output in the same order, to the same bits.
 // The ramp nearly cancels on smooth rows (h[0] against the taps next to it), so the order of the sum decides its
 // rounding: the taps beyond kNear, whose sum is small, go through the tiles, and the near ones are summed outward from
 // h[0] on their own and added last.
-constexpr int kFiltThreads = 256;
-constexpr int kFiltRows = 64, kFiltOut = 256, kFiltK = 64;  // rows and outputs of a block, samples per chunk
-constexpr int kFiltPitch = kFiltRows + 4;
-constexpr int kNear = 15;                                // odd
-constexpr int kFiltStrip = 2 * kFiltOut + 2 * kNear + 2;  // samples around a block's outputs in one row
+constexpr int kFiltThreads = 256, kFiltK = 64;  // samples per chunk
+constexpr int kNear = 15;                       // odd
+// RT rows x OT outputs of one parity per thread; a block's 8 warps lie along the rows, their lanes along the outputs
+template <int RT, int OT>
+struct FiltTile {
+    static constexpr int Rows = 8 * RT, Out = 32 * OT, Pitch = Rows + 4;
+    static constexpr int Strip = 2 * Out + 2 * kNear + 2;  // samples around a block's outputs in one row
+};
+
+// N consecutive floats of shared memory, 4 N (N < 4) or 16 bytes at a time
+template <int N>
+__device__ __forceinline__ void load_floats(const float *p, float *out)
+{
+    if constexpr (N == 2) {
+        const float2 t = *reinterpret_cast<const float2 *>(p);
+        out[0] = t.x, out[1] = t.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(p + i);
+            out[i] = t.x, out[i + 1] = t.y, out[i + 2] = t.z, out[i + 3] = t.w;
+        }
+    }
+}
 
 // The far taps of output n of one row, in the tiles' order, where the tiles' sum is not finite: their zeros for the near
 // taps make NaN of an infinite sample (0 * inf) that only the near sum holds.  q: SDD^2 + v^2 of the row.
@@ -42,19 +62,22 @@ __device__ __noinline__ float far_taps(const KGeom &G, const float *__restrict__
     return sum;
 }
 
-__global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long long rows, const float *__restrict__ proj,
-                                                                float *__restrict__ filt)
+template <int RT, int OT>
+__global__ void __launch_bounds__(kFiltThreads, RT == 8 ? 2 : 4)
+    k_fdk_filter(KGeom G, long long rows, const float *__restrict__ proj, float *__restrict__ filt)
 {
-    constexpr int kWork = 8 * (kFiltOut + kFiltStrip);  // the last step's strips, per warp
-    __shared__ __align__(16) float s_x[kFiltK * kFiltPitch > kWork ? kFiltK * kFiltPitch : kWork];  // [sample][row]
-    __shared__ float s_q[kFiltRows];  // SDD^2 + v^2
-    __shared__ __align__(16) float s_h[kFiltOut + kFiltK];    // taps of the chunk: s_h[i] = tap of j - k = j0 - k0 - K + i
+    using C = FiltTile<RT, OT>;
+    constexpr int V = OT < 4 ? OT : 4;              // taps of one load
+    constexpr int kWork = 8 * (C::Out + C::Strip);  // the last step's strips, per warp
+    __shared__ __align__(16) float s_x[kFiltK * C::Pitch > kWork ? kFiltK * C::Pitch : kWork];  // [sample][row]
+    __shared__ float s_q[C::Rows];  // SDD^2 + v^2
+    __shared__ __align__(16) float s_h[C::Out + kFiltK];    // taps of the chunk: s_h[i] = tap of j - k = j0 - k0 - K + i
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int p = blockIdx.y & 1, j0 = (blockIdx.y >> 1) * kFiltOut;
-    const long long row0 = (long long)blockIdx.x * kFiltRows;
+    const int p = blockIdx.y & 1, j0 = (blockIdx.y >> 1) * C::Out;
+    const long long row0 = (long long)blockIdx.x * C::Rows;
     const float hs = -1.0f / (float)(M_PI * M_PI) * G.inv_du * G.inv_du;
-    if (tid < kFiltRows) {
-        const float v = ((float)((row0 + tid) % G.nv) - G.vc) * G.dv + G.v_off;
+    if (tid < C::Rows) {
+        const float v = ((float)((unsigned)(row0 + tid) % (unsigned)G.nv) - G.vc) * G.dv + G.v_off;
         s_q[tid] = G.sdd * G.sdd + v * v;
     }
     __syncthreads();
@@ -63,74 +86,83 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
         const float u = ((float)i - G.uc) * G.du + G.u_off;
         return __ldg(pr + (long long)r * G.nu + i) * G.sdd * rsqrtf(s_q[r] + u * u);
     };
-    float acc[8][8];  // [row][output]
+    // near taps; the big tile has no registers to keep them
+    constexpr int kTaps = RT == 8 ? 1 : (kNear + 1) / 2;
+    float hn[kTaps];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int i = 0; i < kTaps; ++i) hn[i] = hs / (float)((2 * i + 1) * (2 * i + 1));
+    float acc[RT][OT];  // [row][output]
 #pragma unroll
-        for (int o = 0; o < 8; ++o) acc[r][o] = 0.f;
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int o = 0; o < OT; ++o) acc[r][o] = 0.f;
     const int nk = (G.nu + p) / 2;  // samples of the other parity, 2k + 1 - p < nu
     for (int k0 = 0; k0 < nk; k0 += kFiltK) {
+        // of this chunk; the big tile takes it whole (a bound that is not constant costs it 5 %)
+        const int kend = RT == 8 ? kFiltK : min(kFiltK, (nk - k0 + 15) & ~15);
         __syncthreads();
-        for (int t = tid; t < kFiltRows * kFiltK; t += kFiltThreads) {
+        for (int t = tid; t < C::Rows * kFiltK; t += kFiltThreads) {
             const int k = k0 + t % kFiltK, r = t / kFiltK;
-            s_x[(t % kFiltK) * kFiltPitch + r] = (k < nk && row0 + r < rows) ? weighted(r, 2 * k + 1 - p) : 0.f;
+            if (t % kFiltK < kend)
+                s_x[(t % kFiltK) * C::Pitch + r] = (k < nk && row0 + r < rows) ? weighted(r, 2 * k + 1 - p) : 0.f;
         }
-        for (int t = tid; t < kFiltOut + kFiltK; t += kFiltThreads) {
+        for (int t = tid; t < C::Out + kFiltK; t += kFiltThreads) {
             const float m = (float)(2 * (j0 - k0 - kFiltK + t) + 2 * p - 1);  // odd
             s_h[t] = fabsf(m) <= (float)kNear ? 0.f : hs / (m * m);
         }
         __syncthreads();
-        // output o of the thread at sample k (in the chunk): tap index 8 lane + o + K - k
-        const float *hp = s_h + 8 * lane;
-        float h[12];
+        // output o of the thread at sample k (in the chunk): tap index OT lane + o + K - k
+        const float *hp = s_h + OT * lane;
+        float h[OT + 4];
+        load_floats<OT>(hp + kFiltK, h + 4);
+        for (int kb = 0; kb < kend; kb += 16)
 #pragma unroll
-        for (int i = 0; i < 8; i += 4) {
-            const float4 t = *reinterpret_cast<const float4 *>(hp + kFiltK + i);
-            h[4 + i] = t.x, h[5 + i] = t.y, h[6 + i] = t.z, h[7 + i] = t.w;
-        }
-#pragma unroll 4
-        for (int k = 0; k < kFiltK; k += 4) {  // h[4 + i] = tap index 8 lane + K - k + i
-            const float4 t = *reinterpret_cast<const float4 *>(hp + kFiltK - k - 4);
-            h[0] = t.x, h[1] = t.y, h[2] = t.z, h[3] = t.w;
+            for (int k = kb; k < kb + 16; k += 4) {  // h[4 + i] = tap index OT lane + K - k + i
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float *xp = s_x + (k + q) * kFiltPitch + 8 * warp;
-                const float4 a = *reinterpret_cast<const float4 *>(xp), c = *reinterpret_cast<const float4 *>(xp + 4);
-                const float x[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+                for (int i = 0; i < 4; i += V) load_floats<V>(hp + kFiltK - k - 4 + i, h + i);
 #pragma unroll
-                for (int r = 0; r < 8; ++r)
+                for (int q = 0; q < 4; ++q) {
+                    float x[RT];
+                    load_floats<RT>(s_x + (k + q) * C::Pitch + RT * warp, x);
 #pragma unroll
-                    for (int o = 0; o < 8; ++o) acc[r][o] = fmaf(x[r], h[4 + o - q], acc[r][o]);
+                    for (int r = 0; r < RT; ++r)
+#pragma unroll
+                        for (int o = 0; o < OT; ++o) acc[r][o] = fmaf(x[r], h[4 + o - q], acc[r][o]);
+                }
+#pragma unroll
+                for (int i = OT + 3; i >= 4; --i) h[i] = h[i - 4];
             }
-#pragma unroll
-            for (int i = 11; i >= 4; --i) h[i] = h[i - 4];
-        }
     }
     // a row at a time through shared memory: the near taps from the row's samples around the block's outputs, and
     // stores of neighbouring outputs by neighbouring lanes
     __syncthreads();
     const float h0 = 0.25f * G.inv_du * G.inv_du;
-    float *s_o = s_x + warp * (kFiltOut + kFiltStrip), *s_r = s_o + kFiltOut;
+    float *s_o = s_x + warp * (C::Out + C::Strip), *s_r = s_o + C::Out;
     const int first = 2 * j0 + p - kNear;  // sample of s_r[0]
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int r = 0; r < RT; ++r) {
         __syncwarp();
-        *reinterpret_cast<float4 *>(s_o + 8 * lane) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-        *reinterpret_cast<float4 *>(s_o + 8 * lane + 4) = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
-        const long long row = row0 + 8 * warp + r;
+        if constexpr (OT == 2) {
+            *reinterpret_cast<float2 *>(s_o + OT * lane) = make_float2(acc[r][0], acc[r][1]);
+        } else {
+#pragma unroll
+            for (int o = 0; o < OT; o += 4)
+                *reinterpret_cast<float4 *>(s_o + OT * lane + o) = make_float4(acc[r][o], acc[r][o + 1], acc[r][o + 2], acc[r][o + 3]);
+        }
+        const long long row = row0 + RT * warp + r;
         if (row < rows)
-            for (int t = lane; t < kFiltStrip; t += 32)
-                s_r[t] = (first + t >= 0 && first + t < G.nu) ? weighted(8 * warp + r, first + t) : 0.f;
+            for (int t = lane; t < C::Strip; t += 32)
+                s_r[t] = (first + t >= 0 && first + t < G.nu) ? weighted(RT * warp + r, first + t) : 0.f;
         __syncwarp();
         if (row >= rows) continue;
-        for (int o = lane; o < kFiltOut; o += 32) {
+        for (int o = lane; o < C::Out; o += 32) {
             const int n = 2 * (j0 + o) + p;
             const float *c = s_r + 2 * o + kNear;
             float near = h0 * c[0];
 #pragma unroll
-            for (int m = 1; m <= kNear; m += 2) near = fmaf(hs / (float)(m * m), c[-m] + c[m], near);
+            for (int m = 1; m <= kNear; m += 2) near = fmaf(RT == 8 ? hs / (float)(m * m) : hn[m / 2 % kTaps], c[-m] + c[m], near);
             float far = s_o[o];
-            if (!(fabsf(far) <= FLT_MAX)) far = far_taps(G, proj + row * G.nu, s_q[8 * warp + r], hs, n);
+            if (!(fabsf(far) <= FLT_MAX)) far = far_taps(G, proj + row * G.nu, s_q[RT * warp + r], hs, n);
             if (n < G.nu) filt[row * G.nu + n] = G.du * (near + far);
         }
     }
@@ -139,7 +171,7 @@ __global__ void __launch_bounds__(kFiltThreads, 2) k_fdk_filter(KGeom G, long lo
 // Voxel-driven: a thread owns kFdkCH voxels of one (x, y) column, so a view's u, its interpolation weights and its
 // distance weight (which do not depend on z) serve all of them; a warp covers 8 x 4 columns, whose pixels lie close
 // together whatever the view angle.  Per voxel and view the four gathers remain (10 x 256x256x64, 360 views: 4.4 ->
-// 1.56 ms against a thread per voxel and warps of 32 x 1).
+// 1.49 ms against a thread per voxel and warps of 32 x 1).
 constexpr int kFdkCH = 8;
 
 __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restrict__ views,
@@ -203,13 +235,33 @@ __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restr
 
 }  // namespace
 
+template <int RT, int OT>
+static void launch_filter(const KGeom &kg, long long rows, const float *proj, float *filt, cudaStream_t st)
+{
+    using C = FiltTile<RT, OT>;
+    const int halves = ((kg.nu + 1) / 2 + C::Out - 1) / C::Out;  // tiles of the outputs of one parity
+    k_fdk_filter<RT, OT><<<dim3((unsigned)((rows + C::Rows - 1) / C::Rows), 2 * halves), kFiltThreads, 0, st>>>(kg, rows, proj,
+                                                                                                                filt);
+}
+
+// The small tile where its estimated time is the shorter: 1e7 products a microsecond, against 16.5 us for each chunk of 64
+// samples and wave of big tiles (two on each of the 152 SMs).  Big / small, us: 120 k rows of 64 410 / 144, of 256 688 / 560,
+// of 384 919 / 1141; 11520 of 512 172 / 147, 40 k of 512 415 / 572; 1024 of 1024 100 / 59, 3840 of 1024 140 / 167.
+static bool filter_small(int nu, long long rows)
+{
+    const double small = 0.5 * rows * nu * nu / 1e7;
+    const double big = 16.5 * ceil(nu / 128.0) * ceil((rows + 63) / 64 * 2 * ((nu + 511) / 512) / 304.0);
+    return small < big;
+}
+
 tnlm_status launch_fdk(const KGeom &kg, const ViewGeom *views, const int *view_off, int n_views_total,
                        const float *proj, float *filt, float *vol, cudaStream_t st)
 {
     const long long rows = (long long)n_views_total * kg.nv;
-    const int halves = ((kg.nu + 1) / 2 + kFiltOut - 1) / kFiltOut;  // tiles of the outputs of one parity
-    k_fdk_filter<<<dim3((unsigned)((rows + kFiltRows - 1) / kFiltRows), 2 * halves), kFiltThreads, 0, st>>>(kg, rows, proj,
-                                                                                                            filt);
+    if (filter_small(kg.nu, rows))
+        launch_filter<2, 2>(kg, rows, proj, filt, st);
+    else
+        launch_filter<8, 8>(kg, rows, proj, filt, st);
     TNLM_TRY_CUDA(cudaGetLastError());
     const int nchunks = (kg.nz + kFdkCH - 1) / kFdkCH;
     dim3 grid((kg.nx + 15) / 16, (kg.ny + 7) / 8, nchunks * kg.np);
