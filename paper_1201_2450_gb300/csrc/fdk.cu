@@ -168,27 +168,27 @@ __global__ void __launch_bounds__(kFiltThreads, RT == 8 ? 2 : 4)
     }
 }
 
-// Voxel-driven: a thread owns kFdkCH voxels of one (x, y) column, so a view's u, its interpolation weights and its
+// Voxel-driven: a thread owns CH voxels of one (x, y) column, so a view's u, its interpolation weights and its
 // distance weight (which do not depend on z) serve all of them; a warp covers 8 x 4 columns, whose pixels lie close
 // together whatever the view angle.  Per voxel and view the four gathers remain (10 x 256x256x64, 360 views: 4.4 ->
-// 1.49 ms against a thread per voxel and warps of 32 x 1).
-constexpr int kFdkCH = 8;
-
+// 1.49 ms against a thread per voxel and warps of 32 x 1).  A view of 8 voxels is a chain of gathers behind branches, so
+// small volumes take one voxel per thread (bp_small).
+template <int CH>
 __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restrict__ views,
                                                 const int *__restrict__ view_off, const float *__restrict__ filt,
                                                 float *__restrict__ vol, int nchunks)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ix = (blockIdx.x * 2 + (warp & 1)) * 8 + (lane & 7), iy = (blockIdx.y * 2 + (warp >> 1)) * 4 + (lane >> 3);
-    const int iz0 = (blockIdx.z % nchunks) * kFdkCH, phase = blockIdx.z / nchunks;
+    const int iz0 = (blockIdx.z % nchunks) * CH, phase = blockIdx.z / nchunks;
     if (ix >= G.nx || iy >= G.ny) return;
     const float x = G.b0x + ((float)ix + 0.5f) * G.dx;
     const float y = G.b0y + ((float)iy + 0.5f) * G.dy;
     const int v0 = view_off[phase], v1 = view_off[phase + 1];
     const float wscale = 0.5f * (float)(2.0 * M_PI) / (float)(v1 - v0) * G.sad * G.sdd;
-    float acc[kFdkCH];
+    float acc[CH];
 #pragma unroll
-    for (int k = 0; k < kFdkCH; ++k) acc[k] = 0.f;
+    for (int k = 0; k < CH; ++k) acc[k] = 0.f;
     for (int vg = v0; vg < v1; ++vg) {
         const float c = views[vg].c, s = views[vg].s;
         const float U = G.sad - (x * c + y * s);
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restr
         const float *__restrict__ F = filt + (long long)vg * G.npix;
         const float *__restrict__ Fa = F + ca, *__restrict__ Fb = F + cb;
 #pragma unroll
-        for (int k = 0; k < kFdkCH; ++k) {
+        for (int k = 0; k < CH; ++k) {
             const float z = G.b0z + ((float)(iz0 + k) + 0.5f) * G.dz;
             const float v = G.sdd * z * iU;
             const float fv = (v - G.v_off) * G.inv_dv + G.vc;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128) k_fdk_bp(KGeom G, const ViewGeom *__restr
     }
     const long long base = (long long)phase * G.nvox + ((long long)iz0 * G.ny + iy) * G.nx + ix;
 #pragma unroll
-    for (int k = 0; k < kFdkCH; ++k)
+    for (int k = 0; k < CH; ++k)
         if (iz0 + k < G.nz) vol[base + (long long)k * G.nx * G.ny] = acc[k];
 }
 
@@ -243,6 +243,20 @@ static void launch_filter(const KGeom &kg, long long rows, const float *proj, fl
     k_fdk_filter<RT, OT><<<dim3((unsigned)((rows + C::Rows - 1) / C::Rows), 2 * halves), kFiltThreads, 0, st>>>(kg, rows, proj,
                                                                                                                 filt);
 }
+
+template <int CH>
+static void launch_bp(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *filt, float *vol,
+                      cudaStream_t st)
+{
+    const int nchunks = (kg.nz + CH - 1) / CH;
+    k_fdk_bp<CH><<<dim3((kg.nx + 15) / 16, (kg.ny + 7) / 8, nchunks * kg.np), 128, 0, st>>>(kg, views, view_off, filt, vol,
+                                                                                         nchunks);
+}
+
+// One voxel per thread where runs of 8 are too few threads, or mostly padding.  8 / 1 voxels per thread, 30 views a phase:
+// 4 x 32^3 112 / 24 us, 96x96x48 80 / 48, 4 x 48^3 101 / 50, 96^3 82 / 87, 4 x 64^3 94 / 102, 10 x 64^3 165 / 245;
+// 4 x 512x512x1 225 / 72, 4 x 256x256x3 114 / 76, 4 x 256x256x5 116 / 122.
+static bool bp_small(const KGeom &kg) { return kg.np * kg.nvox < 900000 || kg.nz < 4; }
 
 // The small tile where its estimated time is the shorter: 1e7 products a microsecond, against 16.5 us for each chunk of 64
 // samples and wave of big tiles (two on each of the 152 SMs).  Big / small, us: 120 k rows of 64 410 / 144, of 256 688 / 560,
@@ -263,9 +277,10 @@ tnlm_status launch_fdk(const KGeom &kg, const ViewGeom *views, const int *view_o
     else
         launch_filter<8, 8>(kg, rows, proj, filt, st);
     TNLM_TRY_CUDA(cudaGetLastError());
-    const int nchunks = (kg.nz + kFdkCH - 1) / kFdkCH;
-    dim3 grid((kg.nx + 15) / 16, (kg.ny + 7) / 8, nchunks * kg.np);
-    k_fdk_bp<<<grid, 128, 0, st>>>(kg, views, view_off, filt, vol, nchunks);
+    if (bp_small(kg))
+        launch_bp<1>(kg, views, view_off, filt, vol, st);
+    else
+        launch_bp<8>(kg, views, view_off, filt, vol, st);
     TNLM_TRY_CUDA(cudaGetLastError());
     return TNLM_OK;
 }

@@ -1,6 +1,6 @@
-"""The tiles of the FDK filter (64 rows x 256 outputs, 16 x 64) give the same
-bits: a phase is what it is alone, however many phases share the call and
-choose its tile.  The
+"""The tiles of the FDK filter (64 rows x 256 outputs, 16 x 64) and the runs of
+its backprojection (8 voxels per thread, 1) give the same bits: a phase is what
+it is alone, however many phases share the call and choose its forms.  The
 large call is checked against the FP64 oracle (relative L2 <= 1e-5; without
 noise, as pixel coordinates of long rows carry ~nu 2^-24 pixels of rounding)."""
 import numpy as np
@@ -13,7 +13,7 @@ from paper_1201_2450_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nx,nz,nu,nv,phases", [(20, 7, 510, 80, 50), (20, 7, 395, 90, 100)])
+@pytest.mark.parametrize("nx,nz,nu,nv,phases", [(20, 7, 510, 80, 50), (20, 7, 395, 90, 100), (60, 9, 90, 24, 40), (64, 31, 65, 24, 9)])
 def test_a_phase_alone_equals_a_phase_of_many(ora, nx, nz, nu, nv, phases):
     def desc(n):
         return synth.make_geometry(nx=nx, ny=nx - 2, nz=nz, dx=1.0, nu=nu, nv=nv, du=2.4 * nx / nu, dv=2.0 * nz / nv + 0.1,
