@@ -375,7 +375,7 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
 
 /* Launch-shape autotuning (no counterpart in the paper; it serves speed
  * only).  Several launch shapes of the hot kernels are compiled: projector
- * blocks of {4,8,16} detector columns (the slab walker: 32 x {2,4,8} pixels),
+ * blocks of {4,8,16} warps (the slab walker: 32 x {2,4,8} pixels),
  * band-transpose blocks of 8 x {8,16} voxel columns with 4, or 8 or 16, z
  * cells per thread, and the warp layouts of the box-sum sweep (codes 0 and 2
  * are one, 1 and 3 the other).  Every shape computes each output with the same operations in the
@@ -394,7 +394,8 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
  * The projector shape is 2, 4 or 8 (the slab walker: blocks of 32 x that
  * many detector pixels, one ray per thread, each ray finding all its own
  * crossings) or 102, 104 or 108 (the table walker: blocks of 4, 8 or 16
- * detector columns x 64 rows; the xy cells every detector column crosses are
+ * warps, each of 64 or 32 rows of one detector column or of 16, 8 or 4 rows of
+ * several, by the geometry; the xy cells every detector column crosses are
  * laid out once per handle in device memory, views x nu x (nx + ny + 4,
  * rounded up to even) entries of 8 bytes, and the rows of a column walk them
  * together, adding their own z crossings, over a copy of the volume that

@@ -402,7 +402,8 @@ __device__ __noinline__ float walk_row(const float4 *__restrict__ head, const fl
     return sum;
 }
 
-// A warp walks 32 R rows of one detector column (block: NC adjacent columns), R per lane, 32 apart.
+// A warp walks 32 R rows of one detector column (block: NC adjacent columns), R per lane, 32 apart; R = 0: 2^lr2
+// rows, 4 to 16, of as many adjacent columns as fill the warp (NC times as many in the block).
 // Along an entry's segment e_{k-1} .. e_k a row stays in one voxel unless it crosses a z plane there, once in ~25
 // entries.  The walk takes every entry whole, with the voxel at its end:
 //   acc += (e_k - e_{k-1}) f(c_k, floor z(e_k)),   z(beta) = Ez + beta Gz, 0 outside the volume,
@@ -422,34 +423,39 @@ __device__ __noinline__ float walk_row(const float4 *__restrict__ head, const fl
 // warps: 9.7 ms).
 template <int MODE, int NC, int R, class T>
 __global__ void __launch_bounds__(32 * NC, 32 / NC)
-    k_forward_tab(KGeom G, const ViewGeom *__restrict__ views, const float *__restrict__ vol,
+    k_forward_tab(KGeom G, int lr2, const ViewGeom *__restrict__ views, const float *__restrict__ vol,
                   const T *__restrict__ y, float *__restrict__ out, double *__restrict__ partials)
 {
-    __shared__ float s_acc[32 * R][NC + 1];
+    constexpr bool FEW = R == 0;
+    constexpr int RL = FEW ? 1 : R;
+    const int rows = FEW ? 1 << lr2 : 32;
+    const int nc2 = (NC == 4 ? 2 : (NC == 8 ? 3 : 4)) + (FEW ? 5 - lr2 : 0), ncols = 1 << nc2;  // columns of the block
+    __shared__ float s_acc[32 * RL * (NC + 1)];  // [row][ncols + 1]
     __shared__ double ws[NC];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int row0 = blockIdx.y * 32 * R, vg = blockIdx.z;
+    const int row0 = blockIdx.y * rows * RL, vg = blockIdx.z;
+    const int lane_row = FEW ? lane & (rows - 1) : lane, col = FEW ? (w << (5 - lr2)) + (lane >> lr2) : w;
     const ViewGeom V = views[vg];
-    float acc[R];
+    float acc[RL];
 #pragma unroll
-    for (int j = 0; j < R; ++j) acc[j] = 0.f;
-    const int iu_w = blockIdx.x * NC + w;
+    for (int j = 0; j < RL; ++j) acc[j] = 0.f;
+    const int iu_w = blockIdx.x * ncols + col;
     const float4 *__restrict__ head = reinterpret_cast<const float4 *>(
         G.coltab + coltab_base(vg, iu_w < G.nu ? iu_w : 0, G.coltab_kmax, G.nu));
     const float4 h0 = __ldg(head), h1 = __ldg(head + 1);
     const int K = iu_w < G.nu ? __float_as_int(h1.x) : 0;
-    if (K > 0) {  // the same for the whole warp
+    if (FEW ? __any_sync(0xffffffffu, K > 0) : K > 0) {  // the same for the whole warp
         const float2 *__restrict__ tc = reinterpret_cast<const float2 *>(head) + kColtabHead;  // tc[-1].x: the start
         const float *__restrict__ fp = vol + (long long)V.phase * G.nvox;
         const float fnz = (float)G.nz;
         const float blo = h1.z, bhi = h1.y;
         // where in beta any of the warp's rows is inside the volume (lo, hi), and where all are, by more than rounding
         // could move a voxel (clo, chi)
-        float Ez[R], Gz[R];
+        float Ez[RL], Gz[RL];
         float lo = FLT_MAX, hi = -FLT_MAX, clo = blo, chi = bhi;
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-            const float v = ((float)min(row0 + 32 * j + lane, G.nv - 1) - G.vc) * G.dv + G.v_off;
+        for (int j = 0; j < RL; ++j) {
+            const float v = ((float)min(row0 + 32 * j + lane_row, G.nv - 1) - G.vc) * G.dv + G.v_off;
             Ez[j] = (G.alpha0 * v - G.b0z) * G.inv_dz;
             Gz[j] = v * G.inv_dz;
             const float za = fmaf(blo, Gz[j], Ez[j]), zb = fmaf(bhi, Gz[j], Ez[j]);
@@ -478,7 +484,7 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
         }
         int k0 = 0, k1 = K, c0 = 0, c1 = K;  // entries to walk, and of them those that need no test
         if (!__all_sync(0xffffffffu, clo == blo && chi == bhi)) {
-            for (int o = 16; o > 0; o >>= 1) {
+            for (int o = rows / 2; o > 0; o >>= 1) {
                 lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
                 hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
                 clo = fmaxf(clo, __shfl_xor_sync(0xffffffffu, clo, o));
@@ -491,6 +497,7 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
             c1 = chi < bhi ? min(entry_near(h0, K, chi) - 2, k1) : k1;
             if (!(clo < chi) || c0 >= c1) c0 = c1 = k1;
         }
+        if (FEW && K == 0) k0 = k1 = c0 = c1 = 0;
         // entries k .. end - 1 of the rows; CHECKED: a voxel outside the volume counts 0
         auto walk = [&](int k, int end, auto checked_tag) {
             constexpr bool CHECKED = decltype(checked_tag)::value;
@@ -504,7 +511,7 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
             auto single = [&](int k) {
                 const float2 t = __ldg(tc + k);
 #pragma unroll
-                for (int j = 0; j < R; ++j) acc[j] = fmaf(voxel(t.x, t.y, j), t.x - prev, acc[j]);
+                for (int j = 0; j < RL; ++j) acc[j] = fmaf(voxel(t.x, t.y, j), t.x - prev, acc[j]);
                 prev = t.x;
             };
             if ((k & 1) && k < end) single(k++);
@@ -514,13 +521,13 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
                 const float4 *__restrict__ tp = reinterpret_cast<const float4 *>(tc + k);
                 k += 4 * nb;
                 float4 ta = __ldg(tp), tb = __ldg(tp + 1);
-                float f[4][R], seg[4];
+                float f[4][RL], seg[4];
                 auto request = [&] {
                     const float e[4] = {ta.x, ta.z, tb.x, tb.z}, c[4] = {ta.y, ta.w, tb.y, tb.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int j = 0; j < R; ++j) f[i][j] = voxel(e[i], c[i], j);
+                        for (int j = 0; j < RL; ++j) f[i][j] = voxel(e[i], c[i], j);
                     seg[0] = e[0] - prev;
                     seg[1] = e[1] - e[0];
                     seg[2] = e[2] - e[1];
@@ -533,23 +540,23 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
                 request();
 #pragma unroll 2
                 for (; nb > 1; --nb) {
-                    float f0[4][R], seg0[4];
+                    float f0[4][RL], seg0[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         seg0[i] = seg[i];
 #pragma unroll
-                        for (int j = 0; j < R; ++j) f0[i][j] = f[i][j];
+                        for (int j = 0; j < RL; ++j) f0[i][j] = f[i][j];
                     }
                     request();
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int j = 0; j < R; ++j) acc[j] = fmaf(f0[i][j], seg0[i], acc[j]);
+                        for (int j = 0; j < RL; ++j) acc[j] = fmaf(f0[i][j], seg0[i], acc[j]);
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int j = 0; j < R; ++j) acc[j] = fmaf(f[i][j], seg[i], acc[j]);
+                    for (int j = 0; j < RL; ++j) acc[j] = fmaf(f[i][j], seg[i], acc[j]);
             }
             for (; k < end; ++k) single(k);
         };
@@ -558,20 +565,20 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
         if (c1 < k1) walk(c1, k1, std::true_type{});
     }
 #pragma unroll
-    for (int j = 0; j < R; ++j) s_acc[32 * j + lane][w] = acc[j];
+    for (int j = 0; j < RL; ++j) s_acc[(32 * j + lane_row) * (ncols + 1) + col] = acc[j];
     __syncthreads();
-    // Thread by (row, column) now, NC adjacent columns of a row together: the outputs are written so, and a plane is
+    // Thread by (row, column) now, ncols adjacent columns of a row together: the outputs are written so, and a plane is
     // crossed by adjacent columns in neighbouring cells, by adjacent rows far apart (the gathers of the planes touch
     // ~12 cache lines instead of 32).
     double r2 = 0.0;
 #pragma unroll
-    for (int q = 0; q < R; ++q) {
+    for (int q = 0; q < RL; ++q) {
         const int t = threadIdx.x + 32 * NC * q;
-        const int iv = row0 + t / NC, iu = blockIdx.x * NC + t % NC;
+        const int iv = row0 + (t >> nc2), iu = blockIdx.x * ncols + (t & (ncols - 1));
         if (iv >= G.nv || iu >= G.nu) continue;
         const float u = ((float)iu - G.uc) * G.du + G.u_off;
         const float v = ((float)iv - G.vc) * G.dv + G.v_off;
-        float sum = s_acc[t / NC][t % NC];
+        float sum = s_acc[(t >> nc2) * (ncols + 1) + (t & (ncols - 1))];
         const float4 *__restrict__ head =
             reinterpret_cast<const float4 *>(G.coltab + coltab_base(vg, iu, G.coltab_kmax, G.nu));
         const float4 h1 = __ldg(head + 1);
@@ -631,8 +638,8 @@ __global__ void __launch_bounds__(256) k_zfirst(int nx, int ny, int nz, int ntx,
 size_t volz_bytes(const KGeom &kg) { return (size_t)kg.np * kg.nvox * sizeof(float); }
 
 // Projector launch shape code: 2, 4 or 8 = the slab walker k_forward with blocks of 32 x that
-// many rows; 102, 104 or 108 = the table walker k_forward_tab with blocks of 4, 8 or 16 detector
-// columns, once the handle's column tables exist (else the slab walker with 4 rows).
+// many rows; 102, 104 or 108 = the table walker k_forward_tab with blocks of 4, 8 or 16 warps,
+// once the handle's column tables exist (else the slab walker with 4 rows).
 bool forward_shape_valid(int code)
 {
     return code == 2 || code == 4 || code == 8 || code == 102 || code == 104 || code == 108;
@@ -643,13 +650,65 @@ int forward_shape_in_use(const KGeom &kg)
     return (kg.fwd_by > 100 && !(kg.coltab && kg.volz)) ? 4 : kg.fwd_by;
 }
 
-// Rows per lane of the table walker: two where the detector has them
-static int tab_rows(const KGeom &kg) { return kg.nv <= 32 ? 1 : 2; }
+// The span of depth, within the circle around the volume, in which any ray of the detector rows a .. b is at the volume's
+// height
+struct DepthSpan {
+    double lo, hi;
+    double length() const { return fmax(0.0, hi - lo); }
+};
+
+static DepthSpan rows_span(const KGeom &kg, int a, int b)
+{
+    const double x = fmax(fabs((double)kg.b0x), fabs((double)kg.b0x + (double)kg.nx * kg.dx));
+    const double y = fmax(fabs((double)kg.b0y), fabs((double)kg.b0y + (double)kg.ny * kg.dy));
+    DepthSpan d{kg.sad - hypot(x, y), kg.sad + hypot(x, y)};
+    const double z1 = (double)kg.b0z * kg.sdd, z2 = z1 + (double)kg.nz * kg.dz * kg.sdd;  // v times depth at the two faces
+    const double va = ((double)a - kg.vc) * kg.dv + kg.v_off, vb = ((double)b - kg.vc) * kg.dv + kg.v_off;
+    if (vb > 0) d.lo = fmax(d.lo, z1 / vb);  // some ray above the lower face
+    else if (vb < 0) d.hi = fmin(d.hi, z1 / vb);
+    else if (z1 > 0) d.hi = -1;
+    if (va > 0) d.hi = fmin(d.hi, z2 / va);  // and some below the upper one
+    else if (va < 0) d.lo = fmax(d.lo, z2 / va);
+    else if (z2 < 0) d.hi = -1;
+    return d;
+}
+
+// Rows of a warp of the table walker.  64 (two per lane) cost least per row, but a warp walks all its rows through every
+// entry that any of them has in the volume, with a test where not all have, so few detector rows and volumes that few
+// rows see take fewer rows of several columns.  kCost: a tile of so many rows, relative; with the 1.2 and the 0.2 fitted
+// to the times of all five on 100 scans, where the choice is the best of them or up to 11 % off.  The bits do not depend on
+// it.  64 rows (32 up to 32 detector rows) / the choice, us; before, 32 columns of one row per warp:
+//   128x128x64, 160 views of 256 x 2 pixels 113 / 60 (63), x 4 113 / 60 (65), x 8 114 / 65 (97), x 12 119 / 84 (117);
+//   128x128xnz, 160 views of 256x192, nz = 1 229 / 153 (117), 4 231 / 146 (137), 8 233 / 180 (174), 16 238 / 235 (249);
+//   256x256xnz, 72 views of 512x384, nz = 1 753 / 300 (243), 4 753 / 327 (340), 8 755 / 432 (477), 16 772 / 640 (738).
+int walk_rows(const KGeom &kg)
+{
+    constexpr int kRows[] = {64, 32, 16, 8, 4};
+    constexpr double kCost[] = {178, 141, 90, 56, 36};
+    double best = DBL_MAX;
+    int rows = 64;
+    for (int c = 0; c < 5; ++c) {
+        const int n = kRows[c];
+        double cost = 0.0;
+        for (int a = 0; a < kg.nv; a += n) {
+            const int b = a + n < kg.nv ? a + n : kg.nv;
+            const DepthSpan top = rows_span(kg, a, a), bottom = rows_span(kg, b - 1, b - 1);
+            const double any = rows_span(kg, a, b - 1).length();
+            const double all = DepthSpan{fmax(top.lo, bottom.lo), fmin(top.hi, bottom.hi)}.length();
+            cost += kCost[c] * (0.8 + 0.2 * (b - a) / n) * (any + 1.2 * (any - all));
+        }
+        if (cost < best) {
+            best = cost;
+            rows = n;
+        }
+    }
+    return rows;
+}
 
 static dim3 forward_grid(const KGeom &kg, int code, int n_views)
 {
     if (code < 100) return dim3((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + code - 1) / code, n_views);
-    const int nc = 2 * (code - 100), rows = 32 * tab_rows(kg);
+    const int rows = kg.walk_rows, nc = 2 * (code - 100) * (rows < 32 ? 32 / rows : 1);
     return dim3((kg.nu + nc - 1) / nc, (kg.nv + rows - 1) / rows, n_views);
 }
 
@@ -706,10 +765,13 @@ static void launch_walk(const KGeom &kg, const ViewGeom *views, int n_views, con
                         double *partials, cudaStream_t st)
 {
     const dim3 grid = forward_grid(kg, 100 + NC / 2, n_views);
-    if (tab_rows(kg) == 1)
-        k_forward_tab<MODE, NC, 1, T><<<grid, 32 * NC, 0, st>>>(kg, views, volz, y, out, partials);
+    const int lr2 = kg.walk_rows == 4 ? 2 : (kg.walk_rows == 8 ? 3 : 4);
+    if (kg.walk_rows == 64)
+        k_forward_tab<MODE, NC, 2, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
+    else if (kg.walk_rows == 32)
+        k_forward_tab<MODE, NC, 1, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
     else
-        k_forward_tab<MODE, NC, 2, T><<<grid, 32 * NC, 0, st>>>(kg, views, volz, y, out, partials);
+        k_forward_tab<MODE, NC, 0, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
 }
 
 template <int MODE, int NC, class T>

@@ -37,6 +37,7 @@ struct KGeom {
     // the table walker's FP32 copy of the volume, z fastest: [N_p][ny][nx][nz], written by the
     // projector launch itself (null until built)
     void *volz;
+    int walk_rows;           // rows of a warp of the table walker, 4 to 64 (walk_rows; fixed at creation)
 };
 
 // One projection view: rotation and owning phase.
@@ -84,6 +85,7 @@ bool forward_shape_valid(int code);  // projector launch shape code (KGeom::fwd_
 int forward_shape_in_use(const KGeom &kg);  // the code that runs: the slab walker's 4 without tables
 // column tables of the table walker: entries per view and column (nx + ny - 1 + padding), total, build
 int coltab_kmax(const KGeom &kg);
+int walk_rows(const KGeom &kg);  // the best for the geometry
 size_t coltab_entries(const KGeom &kg, int n_views_total);
 size_t volz_bytes(const KGeom &kg);     // the z-fastest copy of the N_p phases at 4 bytes per voxel
 tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_total, float2 *tab, cudaStream_t st);

@@ -56,3 +56,20 @@ def test_fdk_of_few_rows():
 def test_fdk_of_a_small_volume():
     """32^3 against 64^3: measured 0.37 (1.1 with 8 voxels per thread in both)."""
     assert fdk_us(32, 32, 128, 96, [30] * 4) < 0.6 * fdk_us(64, 64, 128, 96, [30] * 4)
+
+
+def project_us(G):
+    x, p = torch.rand(G.vol_shape, device="cuda"), torch.empty(G.proj_shape, device="cuda")
+    return time_us(lambda: tnlm.tnlm_project(G, x, p))
+
+
+def test_projection_of_few_rows():
+    """2 detector rows against 32: measured 0.39 (0.74 when both filled warps with rows)."""
+    few, many = (project_us(scan(128, 128, 64, 256, nv, [40] * 4, dv=5.6)) for nv in (2, 32))
+    assert few < 0.58 * many
+
+
+def test_projection_of_few_slices():
+    """4 slices under 192 rows against 24: measured 0.59 (0.94 with 64 rows per warp in both)."""
+    few, many = (project_us(scan(128, 128, nz, 256, 192, [40] * 4)) for nz in (4, 24))
+    assert few < 0.77 * many
