@@ -333,25 +333,23 @@ __global__ void __launch_bounds__(32 * NW, bands_warps(CH) / NW)
         const float xc = G.b0x + ((float)ix + 0.5f) * G.dx;
         const float yc = G.b0y + ((float)iy + 0.5f) * G.dy;
         const int v0 = view_off[phase], v_end = view_off[phase + 1];
-        auto add_views = [&](int first) {
-            for (int vg = v0 + first; vg < v_end; vg += ORDER)
-                bands_view<CH, ROWS>(G, s_row, views[vg].c, views[vg].s, xc, yc, iz0, proj + (long long)vg * G.npix,
-                                      pref + (long long)vg * (G.nv + 1) * G.nu, acc);
-        };
-        if (SPLIT > 1 || ORDER == 1) {
-            add_views(SPLIT > 1 ? warp : 0);
-        } else {
-            for (int p = 0; p < ORDER; ++p) {  // a thread reads only what it wrote itself
-                add_views(p);
+        // one loop over the views of all partial sums: with a loop per sum the 16-cell form took 6 % longer
+        int vg = v0 + (SPLIT > 1 ? warp : 0), p = 0;
+        while (vg < v_end) {
+            bands_view<CH, ROWS>(G, s_row, views[vg].c, views[vg].s, xc, yc, iz0, proj + (long long)vg * G.npix,
+                                  pref + (long long)vg * (G.nv + 1) * G.nu, acc);
+            vg += ORDER;
+            if (SPLIT > 1 || ORDER == 1 || vg < v_end) continue;
+            vg = p + 1 < ORDER ? v0 + p + 1 : v_end;
 #pragma unroll
-                for (int k = 0; k < CH; ++k) {
-                    if (p > 0) acc[k] = s_acc[k * NT + tid] + acc[k];
-                    if (p < ORDER - 1) {
-                        s_acc[k * NT + tid] = acc[k];
-                        acc[k] = 0.f;
-                    }
+            for (int k = 0; k < CH; ++k) {  // a thread reads only what it wrote itself
+                if (p > 0) acc[k] = s_acc[k * NT + tid] + acc[k];
+                if (vg < v_end) {
+                    s_acc[k * NT + tid] = acc[k];
+                    acc[k] = 0.f;
                 }
             }
+            ++p;
         }
     }
     if (SPLIT > 1) {
@@ -450,8 +448,9 @@ static long long band_blocks(const KGeom &kg, int np, int ch)
 }
 
 // A launch fills the GPU from about kBandsFill blocks, four resident on each of the 152 SMs; kBandsSplit is where the
-// launches that take their partial sums in turn become the faster ones.
+// launches that take their partial sums in turn become the faster ones, with kBandsViews views a phase or more.
 constexpr long long kBandsFill = 152 * 4, kBandsSplit = 152 * 10;
+constexpr int kBandsViews = 10;
 
 // Cells per thread: chunks of 8 where bp_ch asks for them and the volume has more than 4 slices, as the boundaries
 // beyond the volume cost what the others do (6 x 192x192x1, 30 views of 256x192: 290 us in chunks of 8, 225 of 4; one
@@ -483,15 +482,16 @@ static tnlm_status launch_bands_shape(const KGeom &kg, const ViewGeom *views, co
 // views: stage 37 -> 25 us; 27 us in chunks of 4).  The order depends on the volume alone, not on how many phases the
 // handle holds, so a rank that holds some of a scan's phases gets the bits of a process that holds all.  Partial sums in
 // turn / split, 36 views a phase, by the launch's blocks: 768 (6 of 64x64x32) 175 / 142 us, 1024 (4 of 64^3) 197 / 186,
-// 1280 (10 of 64x64x32) 241 / 219, 1536 (6 of 64^3) 267 / 265, 2304 (4 of 96x96x64) 343 / 378, 2560 (10 of 64^3) 416 / 446.
+// 1280 (10 of 64x64x32) 241 / 219, 1536 (6 of 64^3) 266 / 265, 2304 (4 of 96x96x64) 339 / 378, 2560 (10 of 64^3) 411 / 446;
+// 4 of 64^3 by views: 1 28 / 36, 4 45 / 46, 9 66 / 72, 12 82 / 81, 60 315 / 294.
 template <class T>
 static tnlm_status launch_bands_by_size(const KGeom &kg, const ViewGeom *views, const int *view_off, const float *src,
                                         const float2 *pref, const T *vin, T *vout, float alpha, float beta,
-                                        cudaStream_t st)
+                                        int n_views_total, cudaStream_t st)
 {
     if (band_blocks(kg, 1, 8) >= kBandsFill)
         return launch_bands_shape<1, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
-    if (band_blocks(kg, kg.np, 8) >= kBandsSplit)
+    if (band_blocks(kg, kg.np, 8) >= (n_views_total >= kBandsViews * kg.np ? kBandsSplit : kBandsFill))
         return launch_bands_shape<4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
     if (band_cells(kg) == 8)
         return launch_bands<8, 4, 4, 4, T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st);
@@ -520,7 +520,7 @@ static tnlm_status launch_backproject_t(const KGeom &kg, const ViewGeom *views, 
             set_error("band transpose shape must be CH in {4, 8} and BY in {2, 4} (got %d, %d)", kg.bp_ch, kg.bp_by);
             return TNLM_ERR_ARG;
         }
-        TNLM_TRY(launch_bands_by_size<T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, st));
+        TNLM_TRY(launch_bands_by_size<T>(kg, views, view_off, src, pref, vin, vout, alpha, beta, n_views_total, st));
         return TNLM_OK;
     }
     const size_t smem = sizeof(float4) * kg.nv + sizeof(float) * kBpCH * kBpBX * kBpBY;

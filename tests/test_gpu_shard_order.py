@@ -2,7 +2,8 @@
 that holds all of them gets from the transpose: the order in which a voxel's
 views are summed must not depend on the number of phases in the handle.  The
 sizes are those where the whole scan and one rank's share launch different
-forms (four warps splitting the views of a patch below 1520 blocks)."""
+forms (four warps splitting the views of a patch below 608 blocks, or below 1520 with
+10 views a phase or more)."""
 import numpy as np
 import pytest
 import torch
@@ -16,6 +17,7 @@ CASES = {  # nx, ny, nz, views of each phase, ranks
     "64^3_over_2": (64, 64, 64, [6, 3, 5, 7, 2, 4, 5, 3], 2),
     "96x90x40_over_6": (96, 90, 40, [5, 6, 9, 2, 3, 4], 6),
     "80x80x40_over_4": (80, 80, 40, [4, 5, 6, 1, 7, 3, 2, 2], 4),
+    "64^3_10_views": (64, 64, 64, [12, 11, 16, 14, 12, 9, 15], 2),
     "ragged_16_cells": (88, 61, 70, [5, 2, 6, 4, 3, 8, 1], 7),
 }
 
