@@ -400,8 +400,11 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
  * rounded up to even) entries of 8 bytes, and the rows of a column walk them
  * together, adding their own z crossings, over a copy of the volume that
  * each projection first writes into the handle's workspace z-fastest: N_p x
- * ny x nx x nz voxels of 4 bytes, FP32 also for 16-bit storage; volumes of
- * more than 2^20 slices run the slab walker).  A new handle starts at 104; its tables are built,
+ * ny x nx x nz voxels of 4 bytes, FP32 also for 16-bit storage.  Where rays
+ * cross many thin slices per xy cell, or the volume has more than 2^20, a warp
+ * is 32 columns of one row instead, in blocks of 2, 4 or 8 rows, over a copy of
+ * the slices in 4 x 8 bricks: nx and ny rounded up to multiples of 4 and 8).
+ * A new handle starts at 104; its tables are built,
  * synchronising the device, by the first call that projects (or by
  * tnlm_set_launch_shapes), never during a stream capture; if the tables or
  * the copy cannot be allocated the slab walker with 4 rows runs.  The two

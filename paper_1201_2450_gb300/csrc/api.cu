@@ -65,21 +65,17 @@ static tnlm_status dev_alloc(T **p, size_t count)
 void ensure_coltab(tnlm_geometry *g)
 {
     if (g->d_coltab || g->coltab_failed || g->kg.fwd_by < 100) return;
-    if (g->kg.nz > (1 << 20)) {  // the table walker holds z cells in a float's low bits
-        g->coltab_failed = true;
-        return;
-    }
     const size_t n = coltab_entries(g->kg, g->n_views_total);
     auto give_up = [g] {
         cudaGetLastError();
         cudaFree(g->d_coltab);
-        cudaFree(g->d_volz);
+        cudaFree(g->d_copy);
         g->d_coltab = nullptr;
-        g->d_volz = nullptr;
+        g->d_copy = nullptr;
         g->coltab_failed = true;
     };
     if (forced_alloc_failure() || cudaMalloc(reinterpret_cast<void **>(&g->d_coltab), sizeof(float2) * n) != cudaSuccess ||
-        cudaMalloc(&g->d_volz, volz_bytes(g->kg)) != cudaSuccess) {
+        cudaMalloc(&g->d_copy, copy_bytes(g->kg)) != cudaSuccess) {
         give_up();
         return;
     }
@@ -89,7 +85,7 @@ void ensure_coltab(tnlm_geometry *g)
         return;
     }
     g->kg.coltab = g->d_coltab;
-    g->kg.volz = g->d_volz;
+    g->kg.copy = g->d_copy;
 }
 
 tnlm_status ensure_workspace(tnlm_geometry *g, bool need_tmp, long long n_scalars)
@@ -312,8 +308,10 @@ tnlm_status tnlm_create_geometry(const tnlm_geometry_desc *desc, tnlm_geometry *
     k.bp_ch = 8;
     k.fwd_by = 104;  // the table projector once its tables are built (the slab walker until then)
     k.coltab = nullptr;
+    k.by_columns = walk_by_columns(k);
     k.coltab_kmax = coltab_kmax(k);
-    k.volz = nullptr;
+    k.copy = nullptr;
+    k.brick_slice = brick_slice(d.nx, d.ny);
     k.walk_rows = walk_rows(k);
     g->n_views_total = (int)total;
     g->n_views.assign(d.n_views, d.n_views + d.n_phases);
@@ -358,7 +356,7 @@ void tnlm_destroy_geometry(tnlm_geometry *g)
     cudaFree(g->d_scalars);
     cudaFree(g->d_pref);
     cudaFree(g->d_coltab);
-    cudaFree(g->d_volz);
+    cudaFree(g->d_copy);
     for (cudaEvent_t e : g->phase_ready) cudaEventDestroy(e);
     if (g->copy_start) cudaEventDestroy(g->copy_start);
     if (g->copy_stream) cudaStreamDestroy(g->copy_stream);

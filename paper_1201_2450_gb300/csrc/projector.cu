@@ -168,13 +168,19 @@ __global__ void __launch_bounds__(kFwdBX *BY)
 // the detector row), so every row of the column crosses the same xy cells at
 // the same ray parameters.  k_coltab lays out that sequence once per
 // geometry handle -- entry k of (view, column): the ray parameter where the
-// ray leaves its k-th xy cell, and the offset of that cell's z run -- and
-// k_forward_tab walks the rows of a column through its entries together: a
-// warp is 32 adjacent rows of one column, so an entry is one value for the
-// whole warp and the rows' voxels are neighbours in z.  The walker reads a
-// copy of the volume stored z-fastest, which k_zfirst writes at the start of
-// each projection: 32 rows span a few voxels of one z run, one or two sectors
-// per gather where a row of 32 columns touched three cache lines.
+// ray leaves its k-th xy cell, and the offset of that cell in a copy of the
+// volume that each projection writes first.  Two walks, one of them per
+// handle (walk_by_columns):
+//   k_forward_tab walks the rows of a column through its entries together: a
+//   warp is 32 adjacent rows of one column, so an entry is one value for the
+//   whole warp and the rows' voxels are neighbours in z.  Its copy is stored
+//   z-fastest (k_zfirst): 32 rows span a few voxels of one z run, one or two
+//   sectors per gather where a row of 32 columns touched three cache lines.
+//   k_forward_cols walks 32 adjacent columns of one row, each lane through its
+//   own column's entries (tables interleaved by column), with the row's z
+//   crossings in place.  Its copy holds the z slices in 4 x 8 (x, y) bricks of
+//   32 voxels (k_brick).  It costs more per voxel, but nothing for rows that
+//   miss the volume or do not exist, and less per z plane.
 // ---------------------------------------------------------------------------
 
 constexpr int kColtabHead = 4;  // float2 before a column's entries: what the walk needs of the column, and its start
@@ -188,6 +194,15 @@ constexpr int kColtabAhead = 16;  // room after the last column: the walk reads 
 __host__ __device__ __forceinline__ long long coltab_base(int vg, int iu, int kmax, int nu)
 {
     return ((long long)vg * nu + iu) * kmax;
+}
+
+// The column walk's tables: entries in pairs, pair j of column iu of view vg holds entries 2j, 2j+1 as one float4 at
+// float4 index (vg * kmax / 2 + j) * nu + iu (kmax even), so a warp's lanes read adjacent pairs.  No head.
+constexpr int kPairPad = 3;  // exit entry repeated after the last so reads ahead need no test
+
+__host__ __device__ __forceinline__ long long pair_slot(int vg, int e, int iu, int kmax, int nu)
+{
+    return (((long long)vg * (kmax >> 1) + (e >> 1)) * nu + iu) * 2 + (e & 1);
 }
 
 // The in-plane part of the ray of detector column iu of view V (the same
@@ -251,6 +266,12 @@ struct ColumnRay {
     {
         return ((xa ? ib : ia) * G.nx + (xa ? ia : ib)) * G.nz;
     }
+    // offset of cell (a, b) in a bricked z slice
+    __device__ __forceinline__ int brick_cell(const KGeom &G, int ia, int ib) const
+    {
+        const int x = xa ? ia : ib, y = xa ? ib : ia;
+        return (((y >> 3) * ((G.nx + 3) >> 2) + (x >> 2)) << 5) + ((y & 7) << 2) + (x & 3);
+    }
     // entries of the column: one per interior plane crossed, and the exit
     __device__ __forceinline__ int entries() const { return ok ? n_a + n_b + 1 : 0; }
 };
@@ -259,7 +280,9 @@ struct ColumnRay {
 // t-th plane crossing (a-planes first, then b-planes) at its rank in the merged
 // order, found by binary search over the other axis (ties: the a-plane first);
 // the thread with t == n_a + n_b writes the exit, thread 0 the head.
-// kmax = kColtabHead + nx + ny - 1 + kColtabPad rounded up to an even count.
+// kmax = kColtabHead + nx + ny - 1 + kColtabPad rounded up to an even count, or nx + ny - 1 + kPairPad (COLS: the
+// column walk's tables).
+template <bool COLS>
 __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restrict__ views, float2 *__restrict__ tab,
                                                 int kmax)
 {
@@ -268,7 +291,7 @@ __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restr
     ColumnRay R;
     R.init(G, views[vg], iu);
     float2 *col = tab + coltab_base(vg, iu, kmax, G.nu);
-    if (t == 0) {
+    if (!COLS && t == 0) {
         col[0] = make_float2(R.ok ? fabsf(R.Ga) : 0.f, R.ok ? (R.sa > 0 ? R.Ea - (float)R.ia0 : (float)(R.ia0 + 1) - R.Ea) : 0.f);
         col[1] = make_float2(R.ok ? fabsf(R.Gb) : 0.f, R.ok ? (R.sb > 0 ? R.Eb - (float)R.ib0 : (float)(R.ib0 + 1) - R.Eb) : 0.f);
         col[2] = make_float2(__int_as_float(R.entries()), R.bhi);
@@ -310,7 +333,15 @@ __global__ void __launch_bounds__(128) k_coltab(KGeom G, const ViewGeom *__restr
         cb = R.ib0 + R.sb * k;
     }
     // the cell before this crossing; the crossing clamped to the column's extent
-    col[kColtabHead + e] = make_float2(fminf(fmaxf(beta, R.blo), R.bhi), __int_as_float(R.cell(G, ca, cb)));
+    const float end = fminf(fmaxf(beta, R.blo), R.bhi);
+    if (!COLS) {
+        col[kColtabHead + e] = make_float2(end, __int_as_float(R.cell(G, ca, cb)));
+    } else {
+        const float2 ent = make_float2(end, __int_as_float(R.brick_cell(G, ca, cb)));
+        tab[pair_slot(vg, e, iu, kmax, G.nu)] = ent;
+        if (t == R.n_a + R.n_b)
+            for (int q = 1; q <= kPairPad; ++q) tab[pair_slot(vg, e + q, iu, kmax, G.nu)] = ent;
+    }
 }
 
 constexpr float kCellMagic = 12582912.0f;  // 1.5 * 2^23: one unit per ulp, so z + kCellMagic rounded down holds floor(z)
@@ -607,6 +638,186 @@ __global__ void __launch_bounds__(32 * NC, 32 / NC)
     }
 }
 
+// The column walk.  One ray per thread (block: 32 adjacent columns x BY rows of one view), walked
+// through its column's table two entries per step, the next two entries in
+// flight while the current pair is summed; a z crossing splits an entry's
+// segment (the loop takes any number of them, so no geometry condition
+// applies).
+// Launch bounds: 64 warps per SM (the walk is latency-bound on its voxel gathers, and full occupancy at 32
+// registers, with a few bytes spilled, beats 48 warps at 40 registers by 5 %).
+// vol: the bricked FP32 copy (widened from 16-bit storage by k_brick); y: the stored measurements.
+template <int MODE, int BY, class T>
+__global__ void __launch_bounds__(kFwdBX *BY, 64 / BY)
+    k_forward_cols(KGeom G, const ViewGeom *__restrict__ views, const float *__restrict__ vol,
+                  const T *__restrict__ y, float *__restrict__ out, double *__restrict__ partials)
+{
+    __shared__ double ws[BY];
+    const int iu = blockIdx.x * kFwdBX + threadIdx.x;
+    const int iv = blockIdx.y * BY + threadIdx.y;
+    const int vg = blockIdx.z;
+    double r2 = 0.0;
+    if (iu < G.nu && iv < G.nv) {
+        const ViewGeom V = views[vg];
+        ColumnRay R;
+        R.init(G, V, iu);
+        const float v = ((float)iv - G.vc) * G.dv + G.v_off;
+        const float Dz = v;
+        const float len = sqrtf(R.Dx * R.Dx + R.Dy * R.Dy + Dz * Dz);
+        const float Ez = (G.alpha0 * v - G.b0z) * G.inv_dz;
+        const float Gz = Dz * G.inv_dz;
+        float blo = R.blo, bhi = R.bhi;
+        bool ok = R.ok;
+        slab_grid(Ez, Gz, G.nz, blo, bhi, ok);
+        float acc = 0.f;
+        if (ok && blo < bhi) {
+            const int sc = Gz > 0.f ? 1 : -1;
+            const float ivc = Gz != 0.f ? 1.0f / Gz : 0.f, oc = -Ez * ivc, scf = (float)sc;
+            const int ic0 = clamp_floor(fmaf(blo, Gz, Ez), G.nz), ic1 = clamp_floor(fmaf(bhi, Gz, Ez), G.nz);
+            int nzc = Gz != 0.f ? abs(ic1 - ic0) : 0;  // z planes crossed inside the volume
+            float fc = (float)(ic0 + (Gz > 0.f));
+            float bc = nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
+            const long long zstep = sc * G.brick_slice;  // vol: the bricked copy
+            const float *__restrict__ fp = vol + ((long long)V.phase * G.nz + ic0) * G.brick_slice;
+            const long long st = G.nu;  // pair stride in the interleaved tables
+            const float2 *__restrict__ tc = G.coltab + pair_slot(vg, 0, iu, G.coltab_kmax, G.nu);
+            auto entry_x = [&](int e) { return __ldg(tc + (long long)(e >> 1) * 2 * st + (e & 1)).x; };
+            const int K = R.entries();
+            // this row's entries: the first that ends after blo .. the first that ends at or after bhi
+            // (rows inside the volume's z range enter and leave through its sides: all entries)
+            int k0 = 0, k1 = K - 1;
+            if (blo > R.blo) {
+                int lo = 0, hi = K - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (entry_x(mid) > blo) hi = mid;
+                    else lo = mid + 1;
+                }
+                k0 = lo;
+            }
+            if (bhi < R.bhi) {
+                int lo = k0, hi = K - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (entry_x(mid) >= bhi) hi = mid;
+                    else lo = mid + 1;
+                }
+                k1 = lo;
+            }
+            float bcur = blo;
+            // one table entry (end e, cell offset c): its z crossings, then the rest of its segment
+            auto segment = [&](float e, float c) {
+                float f = ldg_v(fp + __float_as_int(c));
+                while (bc < e) {
+                    acc = fmaf(f, bc - bcur, acc);
+                    bcur = bc;
+                    fp += zstep;
+                    f = ldg_v(fp + __float_as_int(c));
+                    fc += scf;
+                    bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
+                }
+                acc = fmaf(f, e - bcur, acc);
+                bcur = e;
+            };
+            // entries before k1 end before bhi (the tables ascend), so only the last entry is clamped to
+            // the row's exit
+            const float4 *__restrict__ tp = reinterpret_cast<const float4 *>(tc) + (long long)(k0 >> 1) * st;
+            float4 t = __ldg(tp);
+            int k = k0;
+            if ((k & 1) && k < k1) {  // the first entry is the second of its pair
+                segment(t.z, t.w);
+                ++k;
+                tp += st;
+                t = __ldg(tp);
+            }
+            for (; k + 1 < k1; k += 2) {  // pairs of entries strictly before k1, the next pair in flight
+                tp += st;
+                const float4 n = __ldg(tp);
+                float f0 = ldg_v(fp + __float_as_int(t.y));
+                float f1 = ldg_v(fp + __float_as_int(t.w));
+                float e = t.x;
+                if (bc < e) {
+                    do {  // z crossings inside entry k's segment
+                        acc = fmaf(f0, bc - bcur, acc);
+                        bcur = bc;
+                        fp += zstep;
+                        f0 = ldg_v(fp + __float_as_int(t.y));
+                        fc += scf;
+                        bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
+                    } while (bc < e);
+                    f1 = ldg_v(fp + __float_as_int(t.w));
+                }
+                acc = fmaf(f0, e - bcur, acc);
+                bcur = e;
+                e = t.z;
+                while (bc < e) {  // z crossings inside entry k+1's segment
+                    acc = fmaf(f1, bc - bcur, acc);
+                    bcur = bc;
+                    fp += zstep;
+                    f1 = ldg_v(fp + __float_as_int(t.w));
+                    fc += scf;
+                    bc = --nzc > 0 ? fmaf(fc, ivc, oc) : FLT_MAX;
+                }
+                acc = fmaf(f1, e - bcur, acc);
+                bcur = e;
+                t = n;
+            }
+            // the last one or two entries: k1 alone (k odd), or k (even) and then k1 if k < k1
+            if (k & 1) {
+                segment(fminf(t.z, bhi), t.w);
+            } else {
+                segment(fminf(t.x, bhi), t.y);
+                if (k < k1) segment(fminf(t.z, bhi), t.w);
+            }
+        }
+        const float pf = acc * len;
+        const long long o = ((long long)vg * G.nv + iv) * G.nu + iu;
+        if (MODE == 0) {
+            out[o] = pf;
+        } else {
+            const float r = pf - ldg_v(y + o);
+            out[o] = r * len;  // scaled residual consumed by the transpose
+            r2 = (double)r * (double)r;
+        }
+    }
+    if (MODE == 1) {
+        const double s = block_sum_warps<BY>(r2, ws);
+        if (threadIdx.x == 0 && threadIdx.y == 0)
+            partials[((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// The bricked copy of the volume: thread t of z slice (phase, z) takes the
+// 4 x 2 voxels x = 4 bx .. 4 bx + 3, y = 2 py, 2 py + 1 and writes them as the
+// 8 consecutive elements they occupy in brick (bx, py / 4) (rows 2 py and
+// 2 py + 1 of a brick are adjacent), in FP32 whatever the stored type (16-bit
+// values are widened once here rather than at every gather of the walk).
+// Elements outside the volume are written as 0 and never read.
+template <class T>
+__global__ void __launch_bounds__(256) k_brick(KGeom G, const T *__restrict__ vol, float *__restrict__ volb)
+{
+    const int nxb = (G.nx + 3) >> 2, nyh = (G.ny + 1) >> 1;
+    const long long per_slice = (long long)nxb * nyh;
+    const long long n = per_slice * G.nz * G.np;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
+         t += (long long)gridDim.x * blockDim.x) {
+        const long long sl = t / per_slice;  // phase * nz + z
+        const int r = (int)(t - sl * per_slice);
+        const int bx = r % nxb, py = r / nxb;
+        const T *src = vol + sl * G.nx * G.ny;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int x = 4 * bx + i, y = 2 * py + j;
+                v[4 * j + i] = (x < G.nx && y < G.ny) ? ld_v(src + (long long)y * G.nx + x) : 0.f;
+            }
+        float *dst = volb + sl * G.brick_slice + ((((long long)(py >> 2) * nxb + bx) << 5) + ((py & 3) << 3));
+        reinterpret_cast<float4 *>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4 *>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 // The z-fastest copy of the volume, [phase][y][x][z] in FP32 whatever the stored type (16-bit values are widened
 // once here rather than at every gather of the walk): tiles of 32 x by 32 z of one (phase, y) through shared memory.
 template <class T>
@@ -635,11 +846,17 @@ __global__ void __launch_bounds__(256) k_zfirst(int nx, int ny, int nz, int ntx,
 
 }  // namespace
 
-size_t volz_bytes(const KGeom &kg) { return (size_t)kg.np * kg.nvox * sizeof(float); }
+long long brick_slice(int nx, int ny) { return (long long)((nx + 3) / 4) * ((ny + 7) / 8) * 32; }
+
+size_t copy_bytes(const KGeom &kg)
+{
+    return (size_t)kg.np * (kg.by_columns ? (size_t)kg.nz * kg.brick_slice : (size_t)kg.nvox) * sizeof(float);
+}
 
 // Projector launch shape code: 2, 4 or 8 = the slab walker k_forward with blocks of 32 x that
-// many rows; 102, 104 or 108 = the table walker k_forward_tab with blocks of 4, 8 or 16 warps,
-// once the handle's column tables exist (else the slab walker with 4 rows).
+// many rows; 102, 104 or 108 = the table walker, once the handle's column tables exist (else the
+// slab walker with 4 rows), with blocks of 4, 8 or 16 warps (k_forward_tab) or of 32 x 2, 4 or 8
+// pixels (k_forward_cols).
 bool forward_shape_valid(int code)
 {
     return code == 2 || code == 4 || code == 8 || code == 102 || code == 104 || code == 108;
@@ -647,7 +864,7 @@ bool forward_shape_valid(int code)
 
 int forward_shape_in_use(const KGeom &kg)
 {
-    return (kg.fwd_by > 100 && !(kg.coltab && kg.volz)) ? 4 : kg.fwd_by;
+    return (kg.fwd_by > 100 && !(kg.coltab && kg.copy)) ? 4 : kg.fwd_by;
 }
 
 // The span of depth, within the circle around the volume, in which any ray of the detector rows a .. b is at the volume's
@@ -705,9 +922,30 @@ int walk_rows(const KGeom &kg)
     return rows;
 }
 
+// The column walk where rays cross more than 0.4 z planes per xy cell on average: settling a plane takes the row walk
+// about twice the column walk's time.  Row / column walk by that ratio, us: 2 x 128x128xnz, 40 views of 256x160 with a
+// half cone of 16 degrees 0.22 258 / 293, 0.33 324 / 313, 0.44 391 / 332, 0.88 650 / 445; 2 x 64x64xnz, of 6 degrees 0.22 95 /
+// 113, 0.44 145 / 132, 1.8 454 / 307.  And beyond 2^20 slices, where the row walk's cells leave a float's low bits.
+bool walk_by_columns(const KGeom &kg)
+{
+    double sum = 0.0;
+    int n = 0;
+    for (int iv = 0; iv < kg.nv; ++iv)
+        if (rows_span(kg, iv, iv).length() > 0.0) {
+            sum += fabs(((double)iv - kg.vc) * kg.dv + kg.v_off);
+            ++n;
+        }
+    const double planes = n ? sum / n / ((double)kg.sdd * kg.dz) : 0.0;          // crossed per mm along the ray's xy path
+    const double cells = 2.0 / M_PI * (1.0 / (double)kg.dx + 1.0 / (double)kg.dy);  // averaged over the directions
+    return kg.nz > (1 << 20) || planes > 0.4 * cells;
+}
+
 static dim3 forward_grid(const KGeom &kg, int code, int n_views)
 {
-    if (code < 100) return dim3((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + code - 1) / code, n_views);
+    if (code < 100 || kg.by_columns) {
+        const int rows = code % 100;
+        return dim3((kg.nu + kFwdBX - 1) / kFwdBX, (kg.nv + rows - 1) / rows, n_views);
+    }
     const int rows = kg.walk_rows, nc = 2 * (code - 100) * (rows < 32 ? 32 / rows : 1);
     return dim3((kg.nu + nc - 1) / nc, (kg.nv + rows - 1) / rows, n_views);
 }
@@ -725,7 +963,10 @@ long long forward_blocks_max(const KGeom &kg, int n_views_total)
     return a > b ? a : b;
 }
 
-int coltab_kmax(const KGeom &kg) { return (kColtabHead + kg.nx + kg.ny - 1 + kColtabPad + 1) & ~1; }
+int coltab_kmax(const KGeom &kg)
+{
+    return (kg.nx + kg.ny - 1 + (kg.by_columns ? kPairPad : kColtabHead + kColtabPad) + 1) & ~1;
+}
 
 size_t coltab_entries(const KGeom &kg, int n_views_total)
 {
@@ -740,7 +981,10 @@ tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_tot
         return TNLM_ERR_ARG;
     }
     dim3 grid((kg.nx + kg.ny + 127) / 128, kg.nu, n_views_total);
-    k_coltab<<<grid, 128, 0, st>>>(kg, views, tab, kmax);
+    if (kg.by_columns)
+        k_coltab<true><<<grid, 128, 0, st>>>(kg, views, tab, kmax);
+    else
+        k_coltab<false><<<grid, 128, 0, st>>>(kg, views, tab, kmax);
     TNLM_TRY_CUDA(cudaGetLastError());
     return TNLM_OK;
 }
@@ -752,35 +996,51 @@ static void launch_forward_by(const KGeom &kg, const ViewGeom *views, int n_view
     k_forward<MODE, BY, T><<<forward_grid(kg, BY, n_views), dim3(kFwdBX, BY), 0, st>>>(kg, views, vol, y, out, partials);
 }
 
-// np phases of vol into the z-fastest copy
+// phases ph .. ph + np - 1 of vol into the walk's copy
 template <class T>
-static void launch_zfirst(const KGeom &kg, int np, const T *vol, float *volz, cudaStream_t st)
+static void launch_copy(const KGeom &kg, int ph, int np, const T *vol, cudaStream_t st)
 {
-    const int ntx = (kg.nx + 31) / 32, ntz = (kg.nz + 31) / 32;
-    k_zfirst<T><<<(unsigned)((long long)ntx * ntz * kg.ny * np), 256, 0, st>>>(kg.nx, kg.ny, kg.nz, ntx, ntz, vol, volz);
+    const T *src = vol + (long long)ph * kg.nvox;
+    float *dst = static_cast<float *>(kg.copy);
+    if (kg.by_columns) {
+        KGeom kb = kg;
+        kb.np = np;
+        const long long n = (long long)((kg.nx + 3) / 4) * ((kg.ny + 1) / 2) * kg.nz * np;
+        const long long nb = (n + 255) / 256;
+        k_brick<T><<<(unsigned)(nb < 152 * 64 ? nb : 152 * 64), 256, 0, st>>>(
+            kb, src, dst + (long long)ph * kg.nz * kg.brick_slice);
+    } else {
+        const int ntx = (kg.nx + 31) / 32, ntz = (kg.nz + 31) / 32;
+        k_zfirst<T><<<(unsigned)((long long)ntx * ntz * kg.ny * np), 256, 0, st>>>(kg.nx, kg.ny, kg.nz, ntx, ntz, src,
+                                                                                  dst + (long long)ph * kg.nvox);
+    }
 }
 
-template <int MODE, int NC, class T>
-static void launch_walk(const KGeom &kg, const ViewGeom *views, int n_views, const float *volz, const T *y, float *out,
-                        double *partials, cudaStream_t st)
+// BY = 2, 4, 8: rows of a block of the column walk, half the warps of one of the row walk
+template <int MODE, int BY, class T>
+static void launch_walk(const KGeom &kg, const ViewGeom *views, int n_views, const T *y, float *out, double *partials,
+                        cudaStream_t st)
 {
-    const dim3 grid = forward_grid(kg, 100 + NC / 2, n_views);
+    constexpr int NC = 2 * BY;
+    const dim3 grid = forward_grid(kg, 100 + BY, n_views);
     const int lr2 = kg.walk_rows == 4 ? 2 : (kg.walk_rows == 8 ? 3 : 4);
-    if (kg.walk_rows == 64)
-        k_forward_tab<MODE, NC, 2, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
+    const float *copy = static_cast<const float *>(kg.copy);
+    if (kg.by_columns)
+        k_forward_cols<MODE, BY, T><<<grid, dim3(kFwdBX, BY), 0, st>>>(kg, views, copy, y, out, partials);
+    else if (kg.walk_rows == 64)
+        k_forward_tab<MODE, NC, 2, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, copy, y, out, partials);
     else if (kg.walk_rows == 32)
-        k_forward_tab<MODE, NC, 1, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
+        k_forward_tab<MODE, NC, 1, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, copy, y, out, partials);
     else
-        k_forward_tab<MODE, NC, 0, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, volz, y, out, partials);
+        k_forward_tab<MODE, NC, 0, T><<<grid, 32 * NC, 0, st>>>(kg, lr2, views, copy, y, out, partials);
 }
 
-template <int MODE, int NC, class T>
+template <int MODE, int BY, class T>
 static void launch_forward_tab(const KGeom &kg, const ViewGeom *views, int n_views, const T *vol, const T *y,
                                float *out, double *partials, cudaStream_t st)
 {
-    float *volz = static_cast<float *>(kg.volz);
-    launch_zfirst<T>(kg, kg.np, vol, volz, st);
-    launch_walk<MODE, NC, T>(kg, views, n_views, volz, y, out, partials, st);
+    launch_copy<T>(kg, 0, kg.np, vol, st);
+    launch_walk<MODE, BY, T>(kg, views, n_views, y, out, partials, st);
 }
 
 template <int MODE, class T>
@@ -790,9 +1050,9 @@ static void launch_forward_mode(const KGeom &kg, const ViewGeom *views, int n_vi
     switch (forward_shape_in_use(kg)) {
     case 2: launch_forward_by<MODE, 2, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     case 8: launch_forward_by<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 102: launch_forward_tab<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 104: launch_forward_tab<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
-    case 108: launch_forward_tab<MODE, 16, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 102: launch_forward_tab<MODE, 2, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 104: launch_forward_tab<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
+    case 108: launch_forward_tab<MODE, 8, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     default: launch_forward_by<MODE, 4, T>(kg, views, n_views_total, vol, y, out, partials, st); break;
     }
 }
@@ -818,7 +1078,7 @@ tnlm_status launch_forward(const KGeom &kg, const ViewGeom *views, int n_views_t
     return launch_forward_t<float>(kg, views, n_views_total, vol, y, out, partials, mode, st);
 }
 
-// One phase's share of a mode-1 projection: phase ph of vol is copied z-fastest (table walker) and views
+// One phase's share of a mode-1 projection: phase ph of vol is copied for the table walker and views
 // [view_lo, view_hi) projected, writing the same rows of out and the same block partials as the
 // whole-volume launch does; the phases of a volume may so be projected as they arrive.
 tnlm_status launch_forward_phase(const KGeom &kg, const ViewGeom *views, int ph, int view_lo, int view_hi,
@@ -834,18 +1094,17 @@ tnlm_status launch_forward_phase(const KGeom &kg, const ViewGeom *views, int ph,
     const long long off = (long long)view_lo * kg.npix;
     const ViewGeom *vw = views + view_lo;
     double *part = partials + blocks_of(forward_grid(kg, code, view_lo));
-    float *volz = static_cast<float *>(kg.volz);
     KGeom kt = kg;
     if (code > 100) {
-        launch_zfirst<float>(kg, 1, vol + (long long)ph * kg.nvox, volz + (long long)ph * kg.nvox, st);
+        launch_copy<float>(kg, ph, 1, vol, st);
         kt.coltab = kg.coltab + (long long)view_lo * kg.coltab_kmax * kg.nu;
     }
     switch (code) {
     case 2: launch_forward_by<1, 2, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
     case 8: launch_forward_by<1, 8, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
-    case 102: launch_walk<1, 4, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
-    case 104: launch_walk<1, 8, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
-    case 108: launch_walk<1, 16, float>(kt, vw, n, volz, y + off, out + off, part, st); break;
+    case 102: launch_walk<1, 2, float>(kt, vw, n, y + off, out + off, part, st); break;
+    case 104: launch_walk<1, 4, float>(kt, vw, n, y + off, out + off, part, st); break;
+    case 108: launch_walk<1, 8, float>(kt, vw, n, y + off, out + off, part, st); break;
     default: launch_forward_by<1, 4, float>(kg, vw, n, vol, y + off, out + off, part, st); break;
     }
     TNLM_TRY_CUDA(cudaGetLastError());

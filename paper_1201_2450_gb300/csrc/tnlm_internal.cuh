@@ -32,11 +32,15 @@ struct KGeom {
     int bp_by;               // band transpose: warps per block, 2 or 4
     int bp_ch;               // band transpose z cells per thread: 4, or 8 (by size 8 or 16)
     // column tables of the table walker (owned by the geometry handle; null until built)
-    const float2 *coltab;    // [views][nu][coltab_kmax]: (ray parameter leaving the xy cell, z run offset bits)
+    const float2 *coltab;    // (ray parameter leaving the xy cell, offset bits of the cell): [views][nu][coltab_kmax],
+                             // by_columns pairs of entries interleaved over nu
     int coltab_kmax;
-    // the table walker's FP32 copy of the volume, z fastest: [N_p][ny][nx][nz], written by the
-    // projector launch itself (null until built)
-    void *volz;
+    // the table walker's FP32 copy of the volume, written by the projector launch itself (null until
+    // built): z fastest, [N_p][ny][nx][nz]; by_columns z slices of 4 x 8 (x, y) bricks of 32 voxels (x
+    // fastest inside a brick, bricks x-major), [N_p][nz][brick_slice]
+    void *copy;
+    int by_columns;          // which walk (walk_by_columns); fixed at creation
+    long long brick_slice;   // ceil(nx / 4) * ceil(ny / 8) * 32
     int walk_rows;           // rows of a warp of the table walker, 4 to 64 (walk_rows; fixed at creation)
 };
 
@@ -87,7 +91,9 @@ int forward_shape_in_use(const KGeom &kg);  // the code that runs: the slab walk
 int coltab_kmax(const KGeom &kg);
 int walk_rows(const KGeom &kg);  // the best for the geometry
 size_t coltab_entries(const KGeom &kg, int n_views_total);
-size_t volz_bytes(const KGeom &kg);     // the z-fastest copy of the N_p phases at 4 bytes per voxel
+bool walk_by_columns(const KGeom &kg);  // the geometry's better walk
+long long brick_slice(int nx, int ny);  // elements of one bricked z slice
+size_t copy_bytes(const KGeom &kg);     // the table walker's copy of the N_p phases
 tnlm_status build_coltab(const KGeom &kg, const ViewGeom *views, int n_views_total, float2 *tab, cudaStream_t st);
 
 // vout = beta * vin + alpha * P^T proj.  scaled: proj already multiplied by
@@ -270,7 +276,7 @@ struct tnlm_geometry {
     double *d_scalars = nullptr;      // reduction results
     float *d_pref = nullptr;          // column prefix sums for the transpose (prefix_floats)
     float2 *d_coltab = nullptr;       // column tables of the table projector (coltab_entries)
-    void *d_volz = nullptr;           // its z-fastest volume copy (volz_bytes)
+    void *d_copy = nullptr;           // its copy of the volume (copy_bytes)
     // host-buffer entry point: a copy stream and one event per phase (created on first use)
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t copy_start = nullptr;
@@ -297,7 +303,7 @@ namespace tnlm {
 // the band-transpose prefix array (nullptr when the geometry does not admit
 // that transpose or the allocation failed).
 tnlm_status ensure_workspace(tnlm_geometry *g, bool need_tmp, long long n_scalars);
-// Column tables of the table projector and its z-fastest volume copy: built and
+// Column tables of the table projector and its copy of the volume: built and
 // allocated on first use (synchronising the device, so never during stream
 // capture); on allocation failure the slab walker runs instead (the same
 // model, FP32 rounding of its own).

@@ -16,9 +16,9 @@ pytestmark = pytest.mark.gpu
 
 def top_slices(nz):
     """A handle and a volume of nz slices of 2^-10 mm whose top face is the plane z = 0, to the bit; row 32 of 65 lies in
-    it, the others fan out by 0.02 mm."""
+    it, the others fan out by 0.01 mm."""
     dz = 2.0**-10
-    G = tnlm.Geometry(synth.make_geometry(nx=3, ny=2, nz=nz, dx=1.0, dz=dz, cz=-0.5 * nz * dz, nu=9, nv=65, du=0.9, dv=0.02,
+    G = tnlm.Geometry(synth.make_geometry(nx=3, ny=2, nz=nz, dx=1.0, dz=dz, cz=-0.5 * nz * dz, nu=9, nv=65, du=0.9, dv=0.01,
                                           sad=300.0, sdd=450.0, n_phases=1, views_per_phase=[3], angle_offset=0.13))
     x = np.broadcast_to(synth.uniform((1, 1, 2, 3), 820), G.vol_shape).copy()
     x[:, 0] = 1e3  # what a read one slice too far finds: the first slice of the next voxel column
