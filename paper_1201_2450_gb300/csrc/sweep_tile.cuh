@@ -89,6 +89,24 @@ __device__ __forceinline__ void add_checked(float2 D, float2 nc2, float c2, bool
     Z = __fadd2_rn(Z, e);
 }
 
+// add_checked without a branch: the same operations, with a scale of 1 where the reference stays.
+__device__ __forceinline__ void add_straight(float2 D, float2 nc2, float c2, bool ok0, bool ok1, float2 v, float2 &mref,
+                                             float2 &N, float2 &Z)
+{
+    float2 a = __ffma2_rn(D, nc2, mref);
+    if (!ok0) a.x = -FLT_MAX;
+    if (!ok1) a.y = -FLT_MAX;
+    const bool mx = a.x > kRescale, my = a.y > kRescale;
+    const float2 sc = make_float2(mx ? ex2(-a.x) : 1.f, my ? ex2(-a.y) : 1.f);
+    const float2 m = __fmul2_rn(D, make_float2(c2, c2));
+    N = __fmul2_rn(N, sc);
+    Z = __fmul2_rn(Z, sc);
+    mref = make_float2(mx ? m.x : mref.x, my ? m.y : mref.y);
+    const float2 e = make_float2(mx ? 1.f : ex2(a.x), my ? 1.f : ex2(a.y));
+    N = __ffma2_rn(e, v, N);
+    Z = __fadd2_rn(Z, e);
+}
+
 // After the first column: the reference of an output whose best match is good enough becomes 0.
 __device__ __forceinline__ void settle(float &mref, float &N, float &Z)
 {
@@ -129,20 +147,31 @@ struct XPair {
         }
     }
 
-    // one direction: res += N / Z of the thread's outputs, [z][y] pairs along x
-    template <bool SAME>
-    static __device__ __forceinline__ void direction(const float2 (&ai)[SZ][SY], const float *s_a, const float *s_v, int l,
+    // The sums and references of a thread's outputs, [z][y] pairs along x
+    struct State {
+        float2 N[BZ][BY], Z[BZ][BY], mref[BZ][BY];
+    };
+
+    // One direction: res += N / Z of the thread's outputs, [z][y] pairs along x.  Returns 0, or, for a block of 16 outputs and
+    // several columns (APART) and a warp that does not settle, stops after the first column and returns the form (kRest, kRestFar) in which
+    // unsettled() is to go on from its state.
+    static constexpr bool APART = BY == 4 && M_ > 1;
+    enum { kWhole, kRest, kRestFar };
+    template <bool SAME, int PART>
+    static __device__ __forceinline__ int direction(const float2 (&ai)[SZ][SY], const float *s_a, const float *s_v, int l,
                                                      int ry, int rz, int x, int yb, int zb, int nx, int ny, int nz,
-                                                     float c2, bool zin, float2 (&res)[BZ][BY])
+                                                     float c2, bool zin, float2 (&res)[BZ][BY], State &state)
     {
         constexpr int S = 2 * M_ + 1;
+        constexpr bool REST = PART != kWhole;
         float2 N[BZ][BY], Z[BZ][BY], mref[BZ][BY];
 #pragma unroll
         for (int k = 0; k < BZ; ++k)
 #pragma unroll
             for (int j = 0; j < BY; ++j) {
-                N[k][j] = Z[k][j] = make_float2(0.f, 0.f);
-                mref[k][j] = make_float2(FLT_MAX, FLT_MAX);
+                N[k][j] = REST ? state.N[k][j] : make_float2(0.f, 0.f);
+                Z[k][j] = REST ? state.Z[k][j] : make_float2(0.f, 0.f);
+                mref[k][j] = REST ? state.mref[k][j] : make_float2(FLT_MAX, FLT_MAX);
             }
         const float2 nc2 = make_float2(-c2, -c2);
         auto column = [&](int dy, int dx, auto check_tag, auto zin_tag) {
@@ -209,7 +238,9 @@ struct XPair {
                         float2 v;
                         if constexpr (SAME) v = aw[q + k + 1][j + 1];
                         else v = vw[q + k][j];
-                        if constexpr (CHECK) {
+                        if constexpr (CHECK && PART == kRestFar) {
+                            add_straight(Dv, nc2, c2, okz && okx0 && oky[j], okz && okx1 && oky[j], v, mref[k][j], N[k][j], Z[k][j]);
+                        } else if constexpr (CHECK) {
                             add_checked(Dv, nc2, c2, okz && okx0 && oky[j], okz && okx1 && oky[j], v, mref[k][j], N[k][j], Z[k][j]);
                         } else {
                             const float2 a = __ffma2_rn(Dv, nc2, okz ? bias[j] : make_float2(-FLT_MAX, -FLT_MAX));
@@ -222,10 +253,11 @@ struct XPair {
             }
         };
         constexpr int kCentre = M_ * S + M_;
-        for (int it = 0; it < S * S; ++it) {  // the first column, and the others of a warp that did not settle
+        // the first column, and the others of a warp that did not settle
+        for (int it = REST ? 1 : 0; it < S * S; ++it) {
             const int c = it == 0 ? kCentre : (it - 1 < kCentre ? it - 1 : it);
             column(c / S - M_, c % S - M_, std::true_type{}, std::false_type{});
-            if (it == 0) {
+            if (!REST && it == 0) {
                 bool ok = true;  // every output of the warp that counts has the reference 0
 #pragma unroll
                 for (int k = 0; k < BZ; ++k)
@@ -237,7 +269,21 @@ struct XPair {
                         ok = ok && (!in || l == 0 || x >= nx || mref[k][j].x == 0.f) &&
                              (!in || l == 15 || x + 1 >= nx || mref[k][j].y == 0.f);
                     }
-                if (__all_sync(0xffffffffu, ok)) {
+                const bool all = __all_sync(0xffffffffu, ok);
+                if (APART && !all) {
+                    float far = 0.f;
+#pragma unroll
+                    for (int k = 0; k < BZ; ++k)
+#pragma unroll
+                        for (int j = 0; j < BY; ++j) {
+                            state.N[k][j] = N[k][j];
+                            state.Z[k][j] = Z[k][j];
+                            state.mref[k][j] = mref[k][j];
+                            far = fmaxf(far, fmaxf(mref[k][j].x, mref[k][j].y));
+                        }
+                    return __any_sync(0xffffffffu, far > 2.f * kRescale && far < FLT_MAX) ? kRestFar : kRest;
+                }
+                if (all) {
                     if (zin) {
                         for (int b = 0; b < S * S; ++b)
                             if (b != kCentre) column(b / S - M_, b % S - M_, std::false_type{}, std::true_type{});
@@ -256,6 +302,44 @@ struct XPair {
                 res[k][j].x -= N[k][j].x / Z[k][j].x;  // the values were staged negated
                 res[k][j].y -= N[k][j].y / Z[k][j].y;
             }
+        return 0;
+    }
+
+    // this thread's patch block of phase i (clamped reads), kept for all offsets
+    template <class T>
+    static __device__ __forceinline__ void patch(float2 (&ai)[SZ][SY], const T *__restrict__ src, int x, int yb, int zb, int nx,
+                                                 int ny, int nz)
+    {
+        const int x0 = clampi(x, nx), x1 = clampi(x + 1, nx);
+#pragma unroll
+        for (int z = 0; z < SZ; ++z)
+#pragma unroll
+            for (int y = 0; y < SY; ++y) {
+                const T *r = src + ((long long)clampi(zb - 1 + z, nz) * ny + clampi(yb - 1 + y, ny)) * nx;
+                ai[z][y] = make_float2(ld(r + x0), ld(r + x1));
+            }
+    }
+
+    template <class T>
+    static __device__ __noinline__ void read_patch(float2 (&ai)[SZ][SY], const T *__restrict__ src, int x, int yb, int zb, int nx,
+                                                   int ny, int nz)
+    {
+        patch(ai, src, x, yb, zb, nx, ny, nz);
+    }
+
+    // The rest of a direction of a warp whose outputs did not all settle.  kRestFar, where some reference lies far above
+    // what settles: tests without a branch, as some output of the warp moves its reference at nearly every candidate.  Out
+    // of line, and with the patch block read again in it and after it, so that the registers of the other warps do not
+    // depend on it.  6 x 128x128x48, noise sigma, M = 3 (tests in line / here): sigma = h 3.54 / 3.34 ms, 10 h 3.78 /
+    // 3.36; the sweep without unsettled warps at 10 x 256x256x64 15.41 / 15.12 ms.  M = 1: 9 columns do not repay the call.
+    template <bool SAME, int PART, class T>
+    static __device__ __noinline__ void unsettled(const T *__restrict__ src, const float *s_a, const float *s_v, int l, int ry,
+                                                  int rz, int x, int yb, int zb, int nx, int ny, int nz, float c2,
+                                                  float2 (&res)[BZ][BY], State &state)
+    {
+        float2 ai[SZ][SY];
+        patch(ai, src, x, yb, zb, nx, ny, nz);
+        direction<SAME, PART>(ai, s_a, s_v, l, ry, rz, x, yb, zb, nx, ny, nz, c2, false, res, state);
     }
 
     template <bool SAME, class T>
@@ -271,19 +355,8 @@ struct XPair {
         const int x = X0 - 1 + 2 * l, yb = Y0 + ry, zb = Z0 + rz;
         const long long nvox = (long long)nx * ny * nz;
         const bool zin = Z0 - M_ >= 0 && Z0 + TZ - 1 + M_ < nz;  // every candidate of the tile lies inside in z
-        // this thread's patch block of phase i (clamped reads), kept for all offsets
         float2 ai[SZ][SY];
-        {
-            const T *src = wsrc + i * nvox;
-            const int x0 = clampi(x, nx), x1 = clampi(x + 1, nx);
-#pragma unroll
-            for (int z = 0; z < SZ; ++z)
-#pragma unroll
-                for (int y = 0; y < SY; ++y) {
-                    const T *r = src + ((long long)clampi(zb - 1 + z, nz) * ny + clampi(yb - 1 + y, ny)) * nx;
-                    ai[z][y] = make_float2(ld(r + x0), ld(r + x1));
-                }
-        }
+        patch(ai, wsrc + i * nvox, x, yb, zb, nx, ny, nz);
         float2 res[BZ][BY];
 #pragma unroll
         for (int k = 0; k < BZ; ++k)
@@ -295,7 +368,16 @@ struct XPair {
             stage<AY, AZ>(s_a, wsrc + jp * nvox, X0, Y0 - 1 - M_, Z0 - 1 - M_, nx, ny, nz, tid);
             if constexpr (!SAME) stage<VY, VZ>(s_v, vals + jp * nvox, X0, Y0 - M_, Z0 - M_, nx, ny, nz, tid);
             __syncthreads();
-            direction<SAME>(ai, s_a, s_v, l, ry, rz, x, yb, zb, nx, ny, nz, c2, zin, res);
+            State state;
+            const int rest = direction<SAME, kWhole>(ai, s_a, s_v, l, ry, rz, x, yb, zb, nx, ny, nz, c2, zin, res, state);
+            if (APART && rest != 0) {
+                const T *src = wsrc + i * nvox;
+                if (rest == kRest)
+                    unsettled<SAME, kRest>(src, s_a, s_v, l, ry, rz, x, yb, zb, nx, ny, nz, c2, res, state);
+                else
+                    unsettled<SAME, kRestFar>(src, s_a, s_v, l, ry, rz, x, yb, zb, nx, ny, nz, c2, res, state);
+                if (dir == 0) read_patch(ai, src, x, yb, zb, nx, ny, nz);
+            }
         }
         const float inv = 1.f / (2.f + mu);
 #pragma unroll
