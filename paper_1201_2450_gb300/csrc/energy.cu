@@ -16,6 +16,7 @@
 // are summed in the same order in both passes, so the two see identical t.
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "tnlm_internal.cuh"
 
@@ -249,11 +250,13 @@ __global__ void __launch_bounds__(kNT) k_wa_G(int nx, int ny, int nz, int ntz, c
 
 // B[k][p] = sum over o in [-d,d]^3 with x = p - o inside the volume of G[k][x];
 // p on the padded grid [-d, n+d)^3, stored at (p + d).  A warp takes 32 - 2d
-// positions of one row and one offset through every z: 2d + 1 coalesced loads
-// a slice, the x sum by shuffles, the z sum from a ring of slice sums (27 loads
-// a position otherwise: 1.17 -> 0.38 ms per phase pair of 95 x 90 x 71, M = 2).
-template <int D>
-__global__ void __launch_bounds__(256) k_wa_B(int nx, int ny, int nz, const float *__restrict__ G, float *__restrict__ B)
+// positions of one row and one offset through every z (CUT: nch runs of len): 2d + 1
+// coalesced loads a slice, the x sum by shuffles, the z sum from a ring of slice
+// sums (27 loads a position otherwise: 1.17 -> 0.38 ms per phase pair of 95 x 90
+// x 71, M = 2).
+template <int D, bool CUT>
+__global__ void __launch_bounds__(256) k_wa_B(int nx, int ny, int nz, int nch, int len, const float *__restrict__ G,
+                                              float *__restrict__ B)
 {
     const int px_n = nx + 2 * D, py_n = ny + 2 * D, pz_n = nz + 2 * D;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -261,16 +264,18 @@ __global__ void __launch_bounds__(256) k_wa_B(int nx, int ny, int nz, const floa
     const int ty = blockIdx.y * 8 + warp;
     if (ty >= py_n) return;
     const int gx = tx - D, gy = ty - D;
-    const float *__restrict__ Gk = G + (long long)blockIdx.z * nx * ny * nz;
-    float *__restrict__ Bk = B + (long long)blockIdx.z * px_n * py_n * pz_n + (long long)ty * px_n + tx;
+    const int k = CUT ? blockIdx.z / nch : blockIdx.z, z0 = CUT ? (blockIdx.z % nch) * len : 0;
+    const int z1 = CUT ? min(z0 + len, pz_n) : pz_n;
+    const float *__restrict__ Gk = G + (long long)k * nx * ny * nz;
+    float *__restrict__ Bk = B + (long long)k * px_n * py_n * pz_n + (long long)ty * px_n + tx;
     const bool in_x = gx >= 0 && gx < nx, out = lane >= D && lane < 32 - D && tx < px_n;
     const int y0 = max(gy - D, 0), y1 = min(gy + D, ny - 1);
     float ring[2 * D + 1];
 #pragma unroll
     for (int i = 0; i <= 2 * D; ++i) ring[i] = 0.f;
-    for (int z = 0; z < pz_n; ++z) {
+    for (int z = CUT ? z0 - 2 * D : 0; z < z1; ++z) {
         float s = 0.f;
-        if (in_x && z < nz) {
+        if (in_x && (!CUT || z >= 0) && z < nz) {
             const float *__restrict__ row = Gk + (long long)z * ny * nx + gx;
             for (int y = y0; y <= y1; ++y) s += __ldg(row + (long long)y * nx);
         }
@@ -283,7 +288,7 @@ __global__ void __launch_bounds__(256) k_wa_B(int nx, int ny, int nz, const floa
         float b = ring[0];
 #pragma unroll
         for (int i = 1; i <= 2 * D; ++i) b += ring[i];
-        if (out) Bk[(long long)z * py_n * px_n] = b;
+        if (out && (!CUT || z >= z0)) Bk[(long long)z * py_n * px_n] = b;
     }
 }
 
@@ -375,13 +380,26 @@ tnlm_status launch_wa_box_gather(int nx, int ny, int nz, int np, int i, int d, i
     const float *ai = a + (long long)i * nvox, *aj = a + (long long)j * nvox;
     const int R = d + M;
     float *side_i = B + (size_t)W * pn + 2 * (size_t)np * nvox, *side_j = side_i + pn;
-    const dim3 grid((nx + 2 * d + 31 - 2 * d) / (32 - 2 * d), (ny + 2 * d + 7) / 8, W);
-    switch (d) {
-    case 0: k_wa_B<0><<<grid, 256, 0, st>>>(nx, ny, nz, G, B); break;
-    case 1: k_wa_B<1><<<grid, 256, 0, st>>>(nx, ny, nz, G, B); break;
-    case 2: k_wa_B<2><<<grid, 256, 0, st>>>(nx, ny, nz, G, B); break;
-    default: k_wa_B<3><<<grid, 256, 0, st>>>(nx, ny, nz, G, B); break;  // check_sweep_args: d <= 3
-    }
+    // z is cut into runs of 8 or more where whole marches are too few blocks (four on each of the 152 SMs), as with a window
+    // of one candidate (4 x 64^3, d = 1, M = 0: call 304 -> 178 us); the sums do not depend on the cuts
+    const int gx = (nx + 2 * d + 31 - 2 * d) / (32 - 2 * d), gy = (ny + 2 * d + 7) / 8, pz = nz + 2 * d;
+    const long long blocks = (long long)gx * gy * W;
+    const int cuts = (int)(blocks < 608 ? 608 / blocks : 1), runs = cuts < (pz + 7) / 8 ? cuts : (pz + 7) / 8;
+    const int len = (pz + runs - 1) / runs, nch = (pz + len - 1) / len;
+    const dim3 grid(gx, gy, W * nch);
+    auto box = [&](auto cut_tag) {
+        constexpr bool CUT = decltype(cut_tag)::value;
+        switch (d) {
+        case 0: k_wa_B<0, CUT><<<grid, 256, 0, st>>>(nx, ny, nz, nch, len, G, B); break;
+        case 1: k_wa_B<1, CUT><<<grid, 256, 0, st>>>(nx, ny, nz, nch, len, G, B); break;
+        case 2: k_wa_B<2, CUT><<<grid, 256, 0, st>>>(nx, ny, nz, nch, len, G, B); break;
+        default: k_wa_B<3, CUT><<<grid, 256, 0, st>>>(nx, ny, nz, nch, len, G, B); break;  // check_sweep_args: d <= 3
+        }
+    };
+    if (nch > 1)
+        box(std::true_type{});
+    else
+        box(std::false_type{});
     TNLM_TRY_CUDA(cudaGetLastError());
     const long long en = (long long)(nx + 2 * R) * (ny + 2 * R) * (nz + 2 * R);
     const unsigned eb = (unsigned)((en + 255) / 256);
