@@ -378,7 +378,8 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
  * blocks of {4,8,16} warps (the slab walker: 32 x {2,4,8} pixels),
  * band-transpose blocks of 8 x {8,16} voxel columns with 4, or 8 or 16, z
  * cells per thread, and the warp layouts of the box-sum sweep (codes 0 and 2
- * are one, 1 and 3 the other).  Every shape computes each output with the same operations in the
+ * are one, 1 and 3 the other; 0 and 1 are timed, for large volumes of FP32
+ * images: the others have one layout).  Every shape computes each output with the same operations in the
  * same order, so results do not depend on the choice.
  * tnlm_autotune times each shape on the handle's problem size (synthetic
  * inputs in stream-ordered scratch, one warm-up and the best of two timed

@@ -1,6 +1,6 @@
 // Launch-shape autotuner: times the compiled launch shapes of the projector
-// (block rows), the band transpose (block rows, z cells per thread) and the
-// box-sum sweep (warp layout, rows per thread) on the caller's problem size
+// (warps or rows of a block), the band transpose (warps of a block, z cells per
+// thread) and the box-sum sweep (warp layout) on the caller's problem size
 // and keeps the fastest.  Every shape computes each output with the same
 // arithmetic in the same order, so the choice changes speed only.
 #include <cfloat>
@@ -111,15 +111,18 @@ struct Scratch {
     }
 };
 
+// shapes that differ: the warp layouts 0 and 1 of large volumes of FP32 images (2 and 3 are the same two), one otherwise
+int distinct_shapes(bool fp32, int nx, int ny, int nz) { return fp32 && !sweep_small(nx, ny, nz) ? 2 : 1; }
+
 float exponent_scale(float h) { return (float)(1.4426950408889634 / (2.0 * (double)h * (double)h)); }
 
-// the fastest box-sum sweep shape for (d, M) on this size; -1 when (d, M) has no box kernel
+// the fastest of the first n box-sum sweep shapes for (d, M) on this size; -1 when (d, M) has no box kernel
 template <class T, class L>
-tnlm_status tune_sweep(L &&launch_shape, Timer &tm, cudaStream_t st, int *best_v)
+tnlm_status tune_sweep(int n, L &&launch_shape, Timer &tm, cudaStream_t st, int *best_v)
 {
     *best_v = -1;
     float best = FLT_MAX;
-    for (int v = 0; v < kBoxShapes; ++v) {
+    for (int v = 0; v < n; ++v) {
         bool has = true;
         float ms = 0.f;
         TNLM_TRY(tm.best_ms(
@@ -218,6 +221,7 @@ tnlm_status tnlm_autotune(tnlm_geometry *geo, const tnlm_params *p, int *choice,
     int v = -1;
     const float c2 = exponent_scale(p->h);
     TNLM_TRY(tune_sweep<float>(
+        distinct_shapes(true, kg.nx, kg.ny, kg.nz),
         [&](int s, cudaError_t *err) {
             return launch_box_shape(s, p->d, p->M, kg.nx, kg.ny, kg.nz, kg.np, 0, kg.np, f, f, f, geo->d_g, c2, p->mu, 1, st,
                                     err);
@@ -252,6 +256,7 @@ tnlm_status tnlm_autotune_sweep(int nx, int ny, int nz, int np, int d, int M, fl
         k_fill_hash_f16<<<1024, 256, 0, st>>>(a, n, 0x4321u, 0.04f);
         TNLM_TRY_CUDA(cudaGetLastError());
         TNLM_TRY(tune_sweep<__half>(
+            distinct_shapes(false, nx, ny, nz),
             [&](int s, cudaError_t *err) {
                 return launch_box_shape_f16(s, d, M, nx, ny, nz, np, 0, np, a, a, a, o, c2, 1.0f, 0, st, err);
             },
@@ -260,6 +265,7 @@ tnlm_status tnlm_autotune_sweep(int nx, int ny, int nz, int np, int d, int M, fl
         uint16_t *a = static_cast<uint16_t *>(sa.p), *o = static_cast<uint16_t *>(so.p);
         TNLM_TRY(fill_bf16(a, n, 0x4321u, 0.04f, st));
         TNLM_TRY(tune_sweep<uint16_t>(
+            distinct_shapes(false, nx, ny, nz),
             [&](int s, cudaError_t *err) {
                 return launch_box_shape_bf16(s, d, M, nx, ny, nz, np, 0, np, a, a, a, o, c2, 1.0f, 0, st, err);
             },
@@ -268,6 +274,7 @@ tnlm_status tnlm_autotune_sweep(int nx, int ny, int nz, int np, int d, int M, fl
         float *a = static_cast<float *>(sa.p), *o = static_cast<float *>(so.p);
         TNLM_TRY(fill(a, n, 0x4321u, 0.04f, st));
         TNLM_TRY(tune_sweep<float>(
+            distinct_shapes(true, nx, ny, nz),
             [&](int s, cudaError_t *err) {
                 return launch_box_shape(s, d, M, nx, ny, nz, np, 0, np, a, a, a, o, c2, 1.0f, 0, st, err);
             },

@@ -19,19 +19,9 @@ __device__ __forceinline__ void stage_clamped(float *dst, const T *__restrict__ 
     }
 }
 
-// ---------------------------------------------------------------------------
-// k_sweep_box: the same sweep with the patch distance evaluated as a
-// separable box sum.  For a fixed window offset delta,
-//   D_delta(x) = sum_{o in [-d,d]^3} s_delta(x + o),
-//   s_delta(z) = (a_i(clamp z) - a_j(clamp(z + delta)))^2,
-// which is the definition of Eq. 3 / Eq. 9 regrouped (clamping depends on z
-// only).  A warp's 32 lanes span x (lanes d .. 31-d are outputs, the others
-// supply the x halo) and sum along x with shuffles; each thread holds a
-// BY x BZ block of outputs in (y, z) and sums along z and y in registers.
-// The images of the neighbour phase are staged in shared memory per
-// direction; the thread's own patch block of phase i stays in registers for
-// all offsets.
-// ---------------------------------------------------------------------------
+// The block: a warp's 32 lanes span x (lanes d .. 31 - d are outputs, the others supply the x halo) and sum along x with
+// shuffles; each thread holds BY x BZ outputs in (y, z) and sums along z and y in registers.  The images of the neighbour
+// phase are staged in shared memory; the thread's own patch block of phase i stays in registers for all offsets.
 template <int D_, int M_, int BY, int BZ, int WY_, int WZ_>
 struct BoxCfg {
     static constexpr int WY = WY_, WZ = WZ_;        // warps per CTA along y and z
@@ -43,25 +33,6 @@ struct BoxCfg {
     static constexpr int VJX = 32 + 2 * M_, VJY = TY + 2 * M_, VJZ = TZ + 2 * M_;
     static constexpr size_t SMEM = sizeof(float) * ((size_t)AJX * AJY * AJZ + (size_t)VJX * VJY * VJZ);
 };
-
-template <int D_>
-__device__ __forceinline__ float xbox(float b)
-{
-    const unsigned F = 0xffffffffu;
-    if constexpr (D_ == 0) {
-        return b;
-    } else if constexpr (D_ == 1) {
-        return __shfl_up_sync(F, b, 1) + b + __shfl_down_sync(F, b, 1);
-    } else if constexpr (D_ == 2) {
-        const float p = b + __shfl_down_sync(F, b, 1);  // b(x) + b(x+1)
-        return __shfl_up_sync(F, p, 2) + p + __shfl_down_sync(F, b, 2);
-    } else {
-        float acc = b;
-#pragma unroll
-        for (int t = 1; t <= D_; ++t) acc += __shfl_up_sync(F, b, t) + __shfl_down_sync(F, b, t);
-        return acc;
-    }
-}
 
 __device__ __forceinline__ float2 shfl_up2(float2 v, int d)
 {

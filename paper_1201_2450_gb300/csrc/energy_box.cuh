@@ -1,7 +1,6 @@
 // The TNLM half of the total energy and its gradient with frozen weights
-// (see energy.cu for the formulas) on the box-sum machinery of the sweep:
-// the same thread layout, the same separable patch sums and therefore the
-// same patch distance for a pair whichever of its two voxels is the output.
+// (see energy.cu for the formulas) on the box-sum machinery of the sweep: the
+// same thread layout and separable patch sums.
 //   pass 0, output x in phase i, candidates in phase i+1, x's own normaliser:
 //     Lambda_i(x) = log2 Z_i(x),
 //     T1_i(x) = sum_delta w (f_i(x) - f_{i+1}(x+delta)),
@@ -9,6 +8,10 @@
 //   pass 1, output x in phase i, candidates y = x+delta in phase i-1, each
 //     weighted by its own normaliser: w = 2^(-t - Lambda_{i-1}(y)) <= 1,
 //     grad_i(x) += T1_i(x) + sum w (f_i(x) - f_{i-1}(y)).
+// The patch sums are associated by the place of the output in its thread's
+// block (y parity, z in its group of 2 or 4), so the distance of a pair in
+// pass 1 equals the one behind Lambda to rounding only: w is off by about
+// t 2^-24 of itself and w <= 1 holds to that.
 // Every pair contributes its own difference f_i(x) - f_j(y), as in the scatter
 // form of the gradient, so no term of size f has to cancel against another:
 // near a fixed point of Eq. 8 (f close to its weighted means) the gradient is

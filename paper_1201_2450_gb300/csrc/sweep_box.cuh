@@ -14,7 +14,8 @@ namespace box {
 // not depend on where in a tile it lies).  kSmall is a smaller block, for volumes that give the big one too few warps
 // (sweep_small).  Measured (ms per sweep, M = 3, FP32; the 1 x 2 x 4 block of y pairs with running references that
 // these replace in front):
-//   d = 1, 10 x 256x256x64: 17.77 -> 15.56 (kBig2 15.80, kSmall 16.3; 1 x 4 x 4 y pairs 15.59); 4 x 32^3: 0.166 ->
+//   d = 1, 10 x 256x256x64: 17.77 -> 15.56 (kBig2 15.80, kSmall 16.3; 1 x 4 x 4 y pairs 15.59; kBig 15.12 since warps
+//     that keep references leave the common path); 4 x 32^3: 0.166 ->
 //     0.229 big, 0.147 small; 4 x 96x90x40: 0.875 -> 0.833, 0.752; 10 x 128x128x48: 3.83 -> 3.44, 3.52.
 //   d = 2, 4 x 512x512x128: 115.4 -> 75.9 (kBig2 76.5, kSmall 82); 4 x 32^3: 0.242 -> 0.32, 0.203; 4 x 96x90x40:
 //     1.59 -> 1.19, 1.10; 10 x 128x128x48: 7.23 -> 4.78, 5.19.
@@ -26,9 +27,9 @@ template <int D_, int M_, Form F> struct TileOf;
 template <int M_> struct TileOf<1, M_, kBig> { using type = XPair<M_, 1, 4, 4, 2, 168>; };
 template <int M_> struct TileOf<1, M_, kBig2> { using type = XPair<M_, 2, 2, 4, 2, 168>; };
 template <int M_> struct TileOf<1, M_, kSmall> { using type = XPair<M_, 2, 2, 2, 2, 128>; };
-template <int M_> struct TileOf<2, M_, kBig> { using type = YBlock<2, M_, 4, 2, 4, 4, 256>; };
-template <int M_> struct TileOf<2, M_, kBig2> { using type = YBlock<2, M_, 2, 2, 4, 4, 256>; };
-template <int M_> struct TileOf<2, M_, kSmall> { using type = YBlock<2, M_, 2, 2, 4, 2, 168>; };
+template <int M_> struct TileOf<2, M_, kBig> { using type = YBlock<M_, 4, 2, 4, 256>; };
+template <int M_> struct TileOf<2, M_, kBig2> { using type = YBlock<M_, 2, 2, 4, 256>; };
+template <int M_> struct TileOf<2, M_, kSmall> { using type = YBlock<M_, 2, 2, 2, 168>; };
 template <int D_, int M_, Form F> using Tile = typename TileOf<D_, M_, F>::type;
 // Values staged apart from the weights' sources take a second image of shared memory and more loads: with d = 1 the
 // smaller block keeps 16 warps per SM and is the faster one for every volume (17.6 against 20.5 ms at 10 x

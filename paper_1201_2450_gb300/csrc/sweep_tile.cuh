@@ -400,10 +400,11 @@ struct XPair {
     }
 };
 
-// Lanes along x (32 - 2d outputs, d halo lanes either side), BY x BZ outputs in (y, z) per thread, pairs along y.
-template <int D_, int M_, int WY_, int WZ_, int BY_, int BZ_, int REGS>
+// d = 2.  Lanes along x (28 outputs, 2 halo lanes either side), 4 x BZ outputs in (y, z) per thread, pairs along y.
+template <int M_, int WY_, int WZ_, int BZ_, int REGS>
 struct YBlock {
-    static constexpr int D = D_, M = M_, BY = BY_, BZ = BZ_, BP = BY / 2;
+    static constexpr int D_ = 2, D = D_, M = M_, BY = 4, BZ = BZ_, BP = BY / 2;
+    static_assert(BZ == 2 || BZ == 4, "z sums of two or four outputs");
     static constexpr int NT = 32 * WY_ * WZ_;
     static constexpr int TX = 32 - 2 * D_, TY = WY_ * BY, TZ = WZ_ * BZ;
     static constexpr int SP = (BY + 2 * D_) / 2, SZ = BZ + 2 * D_;  // y pairs and z rows of the patch block
@@ -428,9 +429,6 @@ struct YBlock {
     static __device__ __forceinline__ float2 xbox(float2 b)  // sums over x - d .. x + d
     {
         const unsigned F = 0xffffffffu;
-        if constexpr (D_ == 1)
-            return __fadd2_rn(__fadd2_rn(make_float2(__shfl_up_sync(F, b.x, 1), __shfl_up_sync(F, b.y, 1)), b),
-                              make_float2(__shfl_down_sync(F, b.x, 1), __shfl_down_sync(F, b.y, 1)));
         const float2 p = __fadd2_rn(b, make_float2(__shfl_down_sync(F, b.x, 1), __shfl_down_sync(F, b.y, 1)));
         const float2 u = make_float2(__shfl_up_sync(F, p.x, 2), __shfl_up_sync(F, p.y, 2));
         const float2 w = make_float2(__shfl_down_sync(F, b.x, 2), __shfl_down_sync(F, b.y, 2));
@@ -491,14 +489,7 @@ struct YBlock {
                     float2 t[SZ];
 #pragma unroll
                     for (int z = 0; z < SZ; ++z) t[z] = __fadd2_rn(ai[z][p], aw[q + z][p]);
-                    if constexpr (D_ == 1) {
-#pragma unroll
-                        for (int k = 0; k < BZ; k += 2) {
-                            const float2 m = __ffma2_rn(t[k + 2], t[k + 2], __fmul2_rn(t[k + 1], t[k + 1]));
-                            b[k][p] = __ffma2_rn(t[k], t[k], m);
-                            b[k + 1][p] = __ffma2_rn(t[k + 3], t[k + 3], m);
-                        }
-                    } else if constexpr (BZ == 2) {
+                    if constexpr (BZ == 2) {
                         const float2 m = __ffma2_rn(t[3], t[3], __fmul2_rn(t[2], t[2]));
                         const float2 q1 = __ffma2_rn(t[1], t[1], __ffma2_rn(t[4], t[4], m));
                         b[0][p] = __ffma2_rn(t[0], t[0], q1);
@@ -516,27 +507,14 @@ struct YBlock {
 #pragma unroll
                 for (int k = 0; k < BZ; ++k) {
                     const bool okz = ZIN || (unsigned)(zb + k + q - M_) < (unsigned)nz;
-                    float2 o[BP];
-                    if constexpr (D_ == 1) {
-#pragma unroll
-                        for (int h = 0; h < BP; ++h) {
-                            const float m = b[k][h].y + b[k][h + 1].x;
-                            o[h] = make_float2(b[k][h].x + m, m + b[k][h + 1].y);
-                        }
-                    } else if constexpr (BY == 2) {
-                        const float m = (b[k][0].y + b[k][1].x) + (b[k][1].y + b[k][2].x);
-                        o[0] = make_float2(b[k][0].x + m, m + b[k][2].y);
-                    } else {
-                        const float core = b[k][1].y + b[k][2].x;
-                        const float q1 = core + (b[k][0].y + b[k][1].x), q2 = core + (b[k][2].y + b[k][3].x);
-                        o[0] = make_float2(b[k][0].x + q1, q1 + b[k][2].y);
-                        o[1] = make_float2(b[k][1].x + q2, q2 + b[k][3].y);
-                    }
+                    const float core = b[k][1].y + b[k][2].x;
+                    const float q1 = core + (b[k][0].y + b[k][1].x), q2 = core + (b[k][2].y + b[k][3].x);
+                    const float2 o[BP] = {make_float2(b[k][0].x + q1, q1 + b[k][2].y), make_float2(b[k][1].x + q2, q2 + b[k][3].y)};
 #pragma unroll
                     for (int h = 0; h < BP; ++h) {
                         const float2 Dv = xbox(o[h]);
                         float2 v;
-                        if constexpr (SAME) v = D_ == 1 ? make_float2(aw[q + k + 1][h].y, aw[q + k + 1][h + 1].x) : aw[q + k + 2][h + 1];
+                        if constexpr (SAME) v = aw[q + k + 2][h + 1];
                         else v = vw[q + k][h];
                         if constexpr (CHECK) {
                             add_checked(Dv, nc2, c2, okz && ok[2 * h], okz && ok[2 * h + 1], v, mref[k][h], N[k][h], Z[k][h]);

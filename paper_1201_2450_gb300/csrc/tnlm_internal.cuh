@@ -220,8 +220,10 @@ bool launch_box_grouped(int d, int M, const GroupSweep *probs, int nprob, long l
                         int sms, cudaStream_t st, cudaError_t *err);
 bool box_grouped_tiles(int d, int M, int nx, int ny, int nz, int np, int *ntx, int *nty, int *ntz, long long *items);
 
-// Volumes that sweep with the smaller block (sweep_box.cuh has both sides' times).  By the volume alone, so that the
-// phases of a sharded or grouped call and every launch shape sum alike.
+// Volumes that sweep with the smaller block.  By the volume alone, so that the phases of a sharded or grouped call and
+// every launch shape sum alike.  Big / small block, us, d = 1, M = 3, FP32: 2 phases of 64^3 383 / 350, 84^3 610 / 569, 96^3
+// 891 / 887; 10 phases 64^3 1435 / 1433, 84^3 2513 / 2510, 96^3 3914 / 4110; d = 2: 2 of 48^3 301 / 183, 84^3 873 / 825, 96^3
+// 1173 / 1304; 10 of 48^3 884 / 835, 84^3 4003 / 3691, 96^3 5523 / 6088.
 __host__ __device__ inline bool sweep_small(int nx, int ny, int nz) { return (long long)nx * ny * nz <= 600000; }
 
 // Box-sum sweep launch shapes: 0 and 2 are one, 1 and 3 the other of two (big volumes, FP32 images; the others have
