@@ -48,20 +48,23 @@ WORKLOAD = ("NCAT-shaped 4D TNLM-R FP32: 10 phases x 256x256x64 @ 2 mm, 36 views
 NCU_TRAFFIC = {
     # single-kernel captures on the 6-phase case of this workload, scaled by 10/6 to its 10 phases; the
     # projector stage is the z-fastest copy plus the table walk, the transpose stage the column scan plus the bands
-    "k_forward": {"bytes_per_launch": int((100.679936e6 + 56.512768e6 + 609.453568e6 + 161.493504e6) * 10 / 6),
-                  "source_sha": "afafaf434505db22"},
-    "k_backproject": {"bytes_per_launch": int((169.892608e6 + 284.578560e6 + 567.618304e6 + 107.038464e6) * 10 / 6),
-                      "source_sha": "17078780a0ef088a"},
-    "k_sweep": {"bytes_per_launch": int((164.065024e6 + 82.683904e6) * 10 / 6), "source_sha": "27cb305836d9ff71"},
+    "k_forward": {"bytes_per_launch": int((100.677632e6 + 56.667392e6 + 608.884224e6 + 161.562624e6) * 10 / 6),
+                  "source_sha": "8cd5d3abdb99f20e"},
+    "k_backproject": {"bytes_per_launch": int((169.897984e6 + 284.478976e6 + 567.479808e6 + 106.988800e6) * 10 / 6),
+                      "source_sha": "a093efcd597b5a6c"},
+    "k_sweep": {"bytes_per_launch": int((227.013888e6 + 89.516800e6) * 10 / 6), "source_sha": "86f49c39f531828b"},
 }
 
 
-def _src_sha(fname: str) -> str:
-    p = os.path.join(ROOT, "paper_1201_2450_gb300", "csrc", fname)
-    return hashlib.sha256(open(p, "rb").read()).hexdigest()[:16]
+def _src_sha(fnames: tuple) -> str:
+    h = hashlib.sha256()
+    for f in fnames:
+        h.update(open(os.path.join(ROOT, "paper_1201_2450_gb300", "csrc", f), "rb").read())
+    return h.hexdigest()[:16]
 
 
-KERNEL_SRC = {"k_forward": "projector.cu", "k_backproject": "transpose.cu", "k_sweep": "sweep_tile.cuh"}
+KERNEL_SRC = {"k_forward": ("projector.cu",), "k_backproject": ("transpose.cu",),
+              "k_sweep": ("sweep_tile.cuh", "sweep_box.cuh", "tnlm_sweep.cu")}
 
 
 def measured_peaks() -> dict:
@@ -175,20 +178,21 @@ def projection_nnz(desc: dict, device="cuda") -> int:
 # plane by one FMA), per in-plane (b) crossing 3 more, per z (c) crossing 7 (its segment and the next
 # z plane); so per ray 12 (1 + |da|) + 3 |db| + 7 |dc| with da, db, dc the cell steps along each axis.
 K1_FLOP_SLAB, K1_FLOP_B, K1_FLOP_C = 12, 3, 7
-# FP32 operations of the table walk (the default projector), counted from its source: per xy-table
-# entry 3 (its segment length and FMA; only a row's last entry is clamped to its exit), per z crossing
-# 6 (its segment length and FMA, the next z plane by an add and one FMA); so per ray
-# 3 (1 + |dx| + |dy|) + 6 |dz|.  The tables themselves are built once per geometry, not per launch.
-K1_TAB_FLOP_ENTRY, K1_TAB_FLOP_C = 3, 6
-# FP32 operations of a band transpose per non-zero of P on this geometry (an FMA counts 2, a min/max
-# or a conversion 1), the unit of work its rate is quoted in: per (column of 8 cells, view, pixel
-# column) 38 for the chord (two slab tests) and the row-map slopes, 12 for the chord midpoint and the
-# first boundary, then 30 per cell boundary (its height, two row images with margins, the band row's
-# split and accumulations, the prefix difference of the full rows), 320 in all, plus ~13 for the
-# column's footprint per view shared by its ~3.5 pixel columns, over the ~38 (ray, cell) pairs that
-# chord serves (about 4.8 detector rows per 2 mm cell).  The kernel itself needs fewer: one row image
-# per boundary, and a chord per 16 cells.
-K2_FLOP_PER_NNZ = 8.5
+# FP32 operations that the table walk (the default projector, rows of a column together) executes,
+# counted from its source (an FMA counts 2, a min/max or a rounded add 1): per xy-table entry and row 5
+# (the row's z at the entry's end, its floor by a rounded add, the accumulation) and half of the segment
+# length that two rows share; per z plane, which is settled after the walk, 22 (the plane and its
+# parameter 6, the entry that holds it 6, two tests 4, the difference, the clamped length and the
+# accumulation 6); so per ray 5.5 (1 + |dx| + |dy|) + 22 |dz|.  The tables themselves are built once
+# per geometry, not per launch.
+K1_TAB_FLOP_ENTRY, K1_TAB_FLOP_C = 5.5, 22
+# FP32 operations that the band transpose executes per non-zero of P on this geometry: per (column of
+# 16 cells, view, pixel column) 47 for the chord (two slab tests), the row-map slopes and the chord's
+# midpoint, then 24 per cell boundary of the 17 (its height 2, its two row images 4, the bounds and the
+# rounding of the first one 4, the row's share 9, the difference to the boundary before 5), 455 in all,
+# plus ~25 for the column's footprint per view shared by its ~3.5 pixel columns, over the ~76 (ray,
+# cell) pairs that chord serves (about 4.8 detector rows per 2 mm cell).
+K2_FLOP_PER_NNZ = 6.1
 
 
 def projection_counts(desc: dict, device="cuda") -> tuple[int, int, int]:
@@ -242,16 +246,14 @@ def projection_counts(desc: dict, device="cuda") -> tuple[int, int, int]:
     return total, flops, flops_tab
 
 
-# FP32 operations per pair evaluation of the sweep (the hot-path analysis's per-unit figure):
-# 3*3*(2d+1) for the box-sum patch distance plus 8 for the weight and the two accumulations
-# (one exp besides).  This is the unit of work, without the sums that outputs share: the kernel
-# executes 16.25 per pair with d = 1 (4 x 2 x 2 outputs: 48 differences, 84 for the z sums, 24 for
-# the y sums, 24 for the x sums, 80 for the weights and accumulations, over 16), so the fraction of
-# the FP32 peak below is not the FMA pipe's utilisation.
+# FP32 operations that the box-sum sweep of large volumes executes per pair evaluation (one ex2
+# besides), sums that outputs share counted once, over a thread's 16 outputs.  d = 1 (2 x 4 x 2 outputs
+# in x, y, z): 48 differences, 84 for the z sums, 24 for the y sums, 24 for the x sums, 80 for the weights
+# and accumulations.  d = 2 (1 x 4 x 4): 64, 152, 36, 48 and 80.
 
 
-def sweep_ops_per_pair(d: int) -> int:
-    return 9 * (2 * d + 1) + 8
+def sweep_ops_per_pair(d: int) -> float:
+    return {1: 260 / 16, 2: 380 / 16}[d]
 
 
 def measure_compute_peaks(tnlm, stream, gpu_index: int) -> dict:
@@ -389,14 +391,15 @@ def run_ours(args, rank, world, local):
     t = NCU_TRAFFIC.get(dom)
     if t and t.get("source_sha") == _src_sha(KERNEL_SRC[dom]) and cfg.n_phases == 10:
         traffic = t["bytes_per_launch"]
-    # the three kernels are bound by FP32 / integer issue, not HBM: roofline against the FP32 peak
+    # the three kernels are bound by FP32 / integer issue, not HBM: roofline against the FP32 peak, by the operations that
+    # the kernels execute
     nnz, k1_slab, k1_tab = projection_counts(pb.geom)
     in_use = tnlm.tnlm_get_launch_shapes(geom)
     k1_table = in_use["projector_rows"] > 100
     work = {"k_forward": k1_tab if k1_table else k1_slab, "k_backproject": K2_FLOP_PER_NNZ * nnz,
             "k_sweep": sweep_ops_per_pair(cfg.d) * sweep_pairs(cfg)}
     peak_t = cpk["fp32_tflops"]
-    alu = {n: {"algorithmic_tflop": round(work[n] / 1e12, 4),
+    alu = {n: {"executed_tflop": round(work[n] / 1e12, 4),
                "achieved_tflops": round(work[n] / (per_launch_ms[n] / 1e3) / 1e12, 3),
                "frac_of_fp32_peak": round(work[n] / (per_launch_ms[n] / 1e3) / 1e12 / peak_t, 4)} for n in names}
     roofline = {"bound": "alu", "kernel": dom, "achieved": alu[dom]["achieved_tflops"], "peak": round(peak_t, 2),
@@ -404,7 +407,7 @@ def run_ours(args, rank, world, local):
                 "peak_source": f"measured FP32 FMA throughput of this GPU ({cpk['sms']} SMs; FFMA "
                                f"{cpk['ffma_tflops']} and packed FFMA2 {cpk['ffma2_tflops']} TFLOP/s, the larger "
                                f"taken; SM clock median {cpk['clocks'].get('sm_mhz')} MHz during the probes)",
-                "work": f"{work[dom]:.4g} FP32 ops per launch (nnz(P) = {nnz:.4g})",
+                "work": f"{work[dom]:.4g} FP32 ops executed per launch (nnz(P) = {nnz:.4g})",
                 "hbm_frac": hbm[dom]["frac_of_hbm"]}
     nvox_upd = cfg.n_phases * cfg.vol[0] * cfg.vol[1] * cfg.vol[2]
     sweep_s = per_launch_ms["k_sweep"] / 1e3
