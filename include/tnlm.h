@@ -396,7 +396,7 @@ tnlm_status tnlm_energy_grad_weights(int nx, int ny, int nz, int n_phases, const
  * many detector pixels, one ray per thread, each ray finding all its own
  * crossings) or 102, 104 or 108 (the table walker: blocks of 4, 8 or 16
  * warps, each of 64 or 32 rows of one detector column or of 16, 8 or 4 rows of
- * several, by the geometry; the xy cells every detector column crosses are
+ * several, by the geometry and the number of views; the xy cells every detector column crosses are
  * laid out once per handle in device memory, views x nu x (nx + ny + 4,
  * rounded up to even) entries of 8 bytes, and the rows of a column walk them
  * together, adding their own z crossings, over a copy of the volume that

@@ -312,7 +312,7 @@ tnlm_status tnlm_create_geometry(const tnlm_geometry_desc *desc, tnlm_geometry *
     k.coltab_kmax = coltab_kmax(k);
     k.copy = nullptr;
     k.brick_slice = brick_slice(d.nx, d.ny);
-    k.walk_rows = walk_rows(k);
+    k.walk_rows = walk_rows(k, (int)total);
     g->n_views_total = (int)total;
     g->n_views.assign(d.n_views, d.n_views + d.n_phases);
     g->angles.assign(d.angles_rad, d.angles_rad + total);

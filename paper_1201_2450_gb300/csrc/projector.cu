@@ -867,18 +867,23 @@ int forward_shape_in_use(const KGeom &kg)
     return (kg.fwd_by > 100 && !(kg.coltab && kg.copy)) ? 4 : kg.fwd_by;
 }
 
-// The span of depth, within the circle around the volume, in which any ray of the detector rows a .. b is at the volume's
-// height
+// Depth within the circle around the volume: all of it (circle_span), and where any ray of the detector rows a .. b is at
+// the volume's height (rows_span)
 struct DepthSpan {
     double lo, hi;
     double length() const { return fmax(0.0, hi - lo); }
 };
 
-static DepthSpan rows_span(const KGeom &kg, int a, int b)
+static DepthSpan circle_span(const KGeom &kg)
 {
     const double x = fmax(fabs((double)kg.b0x), fabs((double)kg.b0x + (double)kg.nx * kg.dx));
     const double y = fmax(fabs((double)kg.b0y), fabs((double)kg.b0y + (double)kg.ny * kg.dy));
-    DepthSpan d{kg.sad - hypot(x, y), kg.sad + hypot(x, y)};
+    return DepthSpan{kg.sad - hypot(x, y), kg.sad + hypot(x, y)};
+}
+
+static DepthSpan rows_span(const KGeom &kg, int a, int b)
+{
+    DepthSpan d = circle_span(kg);
     const double z1 = (double)kg.b0z * kg.sdd, z2 = z1 + (double)kg.nz * kg.dz * kg.sdd;  // v times depth at the two faces
     const double va = ((double)a - kg.vc) * kg.dv + kg.v_off, vb = ((double)b - kg.vc) * kg.dv + kg.v_off;
     if (vb > 0) d.lo = fmax(d.lo, z1 / vb);  // some ray above the lower face
@@ -890,32 +895,40 @@ static DepthSpan rows_span(const KGeom &kg, int a, int b)
     return d;
 }
 
-// Rows of a warp of the table walker.  64 (two per lane) cost least per row, but a warp walks all its rows through every
-// entry that any of them has in the volume, with a test where not all have, so few detector rows and volumes that few
-// rows see take fewer rows of several columns.  kCost: a tile of so many rows, relative; with the 1.2 and the 0.2 fitted
-// to the times of all five on 100 scans, where the choice is the best of them or up to 11 % off.  The bits do not depend on
-// it.  64 rows (32 up to 32 detector rows) / the choice, us; before, 32 columns of one row per warp:
-//   128x128x64, 160 views of 256 x 2 pixels 113 / 60 (63), x 4 113 / 60 (65), x 8 114 / 65 (97), x 12 119 / 84 (117);
-//   128x128xnz, 160 views of 256x192, nz = 1 229 / 153 (117), 4 231 / 146 (137), 8 233 / 180 (174), 16 238 / 235 (249);
-//   256x256xnz, 72 views of 512x384, nz = 1 753 / 300 (243), 4 753 / 327 (340), 8 755 / 432 (477), 16 772 / 640 (738).
-int walk_rows(const KGeom &kg)
+// Rows of a warp of the table walker.  64 (two per lane; 32 where the detector has no more) cost least per row, but a warp
+// walks all its rows through every entry that any of them has in the volume, with a test where not all have, so few detector
+// rows and volumes that few rows see take fewer rows of several columns.  kCost: a tile of so many rows, relative; with the
+// other constants fitted to the times of all five on 170 scans.  Fewer rows are taken where they are estimated at 0.8 of the
+// time or less (they are never more than 1 % slower there) and the launch is more than one wave (32 warps on each of the 152
+// SMs; below that 32 rows have the shorter chain, 12.2 against 13.3 us at 32^3 with 40 views of 64 x 8).  The bits do not
+// depend on the choice.  64 rows (32 up to 32 detector rows) / the choice, us; before, 32 columns of one row per warp:
+//   128x128x64, 160 views of 256 x 2 pixels 113 / 61 (62), x 4 113 / 61 (68), x 8 114 / 65 (95), x 12 119 / 84 (116);
+//   128x128xnz, 160 views of 256x192, nz = 1 228 / 154 (117), 4 230 / 147 (137), 8 232 / 187 (173);
+//   256x256xnz, 72 views of 512x384, nz = 1 750 / 300 (242), 4 750 / 363 (341), 8 752 / 438 (478), 12 760 / 540 (611).
+int walk_rows(const KGeom &kg, int n_views)
 {
     constexpr int kRows[] = {64, 32, 16, 8, 4};
-    constexpr double kCost[] = {178, 141, 90, 56, 36};
-    double best = DBL_MAX;
-    int rows = 64;
+    constexpr double kCost[] = {178, 140, 98, 57, 49};
+    const DepthSpan whole = circle_span(kg);
+    const int usual = kg.nv <= 32 ? 32 : 64;
+    if ((long long)kg.nu * n_views * ((kg.nv + usual - 1) / usual) <= 152 * 32) return usual;
+    double limit = DBL_MAX;  // the estimate to fall below
+    int rows = usual;
     for (int c = 0; c < 5; ++c) {
         const int n = kRows[c];
+        if (n > usual) continue;
         double cost = 0.0;
         for (int a = 0; a < kg.nv; a += n) {
             const int b = a + n < kg.nv ? a + n : kg.nv;
             const DepthSpan top = rows_span(kg, a, a), bottom = rows_span(kg, b - 1, b - 1);
             const double any = rows_span(kg, a, b - 1).length();
             const double all = DepthSpan{fmax(top.lo, bottom.lo), fmin(top.hi, bottom.hi)}.length();
-            cost += kCost[c] * (0.8 + 0.2 * (b - a) / n) * (any + 1.2 * (any - all));
+            if (any > 0.0) cost += kCost[c] * (0.8 + 0.2 * (b - a) / n) * (any + 1.05 * (any - all) + 0.06 * whole.length());
         }
-        if (cost < best) {
-            best = cost;
+        if (n == usual) {
+            limit = 0.8 * cost;
+        } else if (cost < limit) {
+            limit = cost;
             rows = n;
         }
     }

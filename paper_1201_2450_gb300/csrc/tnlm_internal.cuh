@@ -41,7 +41,7 @@ struct KGeom {
     void *copy;
     int by_columns;          // which walk (walk_by_columns); fixed at creation
     long long brick_slice;   // ceil(nx / 4) * ceil(ny / 8) * 32
-    int walk_rows;           // rows of a warp of the table walker, 4 to 64 (walk_rows; fixed at creation)
+    int walk_rows;           // rows of a warp of the table walker, 4 to 64 (walk_rows(); fixed at creation)
 };
 
 // One projection view: rotation and owning phase.
@@ -89,7 +89,7 @@ bool forward_shape_valid(int code);  // projector launch shape code (KGeom::fwd_
 int forward_shape_in_use(const KGeom &kg);  // the code that runs: the slab walker's 4 without tables
 // column tables of the table walker: entries per view and column (nx + ny - 1 + padding), total, build
 int coltab_kmax(const KGeom &kg);
-int walk_rows(const KGeom &kg);  // the best for the geometry
+int walk_rows(const KGeom &kg, int n_views);  // the best for the geometry
 size_t coltab_entries(const KGeom &kg, int n_views_total);
 bool walk_by_columns(const KGeom &kg);  // the geometry's better walk
 long long brick_slice(int nx, int ny);  // elements of one bricked z slice

@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 def scan(nx, nz, nu, nv, **kw):
-    d = dict(dx=1.0, du=1.3, dv=1.1, sad=300.0, sdd=450.0, angle_offset=0.13, n_phases=2, views_per_phase=[3, 2])
+    views = 5000 // nu + 1  # more than one wave of warps, below which there are always 32 or 64 rows
+    d = dict(dx=1.0, du=1.3, dv=1.1, sad=300.0, sdd=450.0, angle_offset=0.13, n_phases=2, views_per_phase=[views - 2, 2])
     d.update(kw)
     return tnlm.Geometry(synth.make_geometry(nx=nx, ny=nx - 3, nz=nz, nu=nu, nv=nv, **d))
 

@@ -15,6 +15,7 @@ def time_us(fn, repeats=7, calls=10):
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     best = float("inf")
     for _ in range(repeats):
+        torch.cuda._sleep(4_000_000)  # ~2 ms: the calls are queued behind it, so that the GPU's time counts and not the host's
         a.record()
         for _ in range(calls):
             fn()
