@@ -48,8 +48,8 @@ WORKLOAD = ("NCAT-shaped 4D TNLM-R FP32: 10 phases x 256x256x64 @ 2 mm, 36 views
 NCU_TRAFFIC = {
     # single-kernel captures on the 6-phase case of this workload, scaled by 10/6 to its 10 phases; the
     # projector stage is the z-fastest copy plus the table walk, the transpose stage the column scan plus the bands
-    "k_forward": {"bytes_per_launch": int((100.677632e6 + 56.667392e6 + 608.884224e6 + 161.562624e6) * 10 / 6),
-                  "source_sha": "8cd5d3abdb99f20e"},
+    "k_forward": {"bytes_per_launch": int((100.672000e6 + 55.544832e6 + 607.070464e6 + 157.668096e6) * 10 / 6),
+                  "source_sha": "90dc4e6827dd2a13"},
     "k_backproject": {"bytes_per_launch": int((169.897984e6 + 284.478976e6 + 567.479808e6 + 106.988800e6) * 10 / 6),
                       "source_sha": "a093efcd597b5a6c"},
     "k_sweep": {"bytes_per_launch": int((227.013888e6 + 89.516800e6) * 10 / 6), "source_sha": "86f49c39f531828b"},
